@@ -153,21 +153,25 @@ dpb_status dpb_plan_create(const dpb_config *cfg, const uint32_t *generators, dp
         return dpb::fail(DPB_ERR_CUDA, "cudaGetDevice or its multiprocessor count failed");
     }
     const size_t mb = sizeof(uint32_t) * p->M.size(), gb = sizeof(uint32_t) * p->G.size();
-    struct Up {
-        uint32_t **dst;
-        const std::vector<uint32_t> *src;
-    } ups[] = {{&p->dM, &p->M}, {&p->dG, &p->G}, {&p->dVH, &p->VH}, {&p->dFRAG, &p->FRAG}, {&p->dDD, &p->DD},
-                {&p->dGT, &p->GT},     {&p->dVH2, &p->VH2}, {&p->dCOSET, &p->COSET}};
+    struct Up {  // every table is of 4-byte words
+        void **dst;
+        const void *src;
+        size_t words;
+    };
+    auto up = [](auto **dst, const auto &src) { return Up{reinterpret_cast<void **>(dst), src.data(), src.size()}; };
+    const Up ups[] = {up(&p->dM, p->M),       up(&p->dG, p->G),   up(&p->dVH, p->VH),
+                      up(&p->dFRAG, p->FRAG), up(&p->dDD, p->DD), up(&p->dGT, p->GT),
+                      up(&p->dVH2, p->VH2),   up(&p->dGF, p->GF), up(&p->dCOSET, p->COSET)};
     for (const Up &u : ups) {
-        if (u.src->empty()) continue;
-        const size_t bytes = sizeof(uint32_t) * u.src->size();
+        if (u.words == 0) continue;
+        const size_t bytes = sizeof(uint32_t) * u.words;
         if (cudaMalloc(u.dst, bytes) != cudaSuccess) {
             cudaGetLastError();
             for (const Up &v : ups) cudaFree(*v.dst);
             delete p;
             return dpb::fail(DPB_ERR_NO_MEMORY, "device table allocation failed");
         }
-        if (cudaMemcpy(*u.dst, u.src->data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
+        if (cudaMemcpy(*u.dst, u.src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
             cudaGetLastError();
             for (const Up &v : ups) cudaFree(*v.dst);
             delete p;
@@ -194,6 +198,7 @@ dpb_status dpb_plan_destroy(dpb_plan *plan) {
     cudaFree(plan->dDD);
     cudaFree(plan->dGT);
     cudaFree(plan->dVH2);
+    cudaFree(plan->dGF);
     cudaFree(plan->dCOSET);
     if (cur >= 0 && cur != plan->device) cudaSetDevice(cur);
     delete plan;

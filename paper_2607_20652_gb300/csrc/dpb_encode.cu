@@ -220,6 +220,8 @@ size_t encode_smem_per_warp(const dpb_plan *p) {
 cudaError_t launch_encode(const dpb_plan *p, const void *x, int64_t T, const float *mu,
                           const float *sigma, int32_t *idx, float *val, float *xnorm,
                           int32_t *status, float2 *tab_scratch, cudaStream_t stream) {
+    // 16 children and beams up to 16 outside the tensor-core encoder's types and widths (fp32 rows above all)
+    if (p->fma_encode) return launch_encode_fma(p, x, T, mu, sigma, idx, val, xnorm, status, stream);
     // standardisation tables as (mu, 1 / sigma) pairs: one load per candidate
     const float2 *tab = nullptr;
     if (mu && tab_scratch) {

@@ -542,22 +542,24 @@ __device__ __forceinline__ bool level0_union(const uint4 *row, int nch, int k, u
     return true;
 }
 
-// Level 0 with standardisation tables: the union path above on 64-bit words
-// of z = (x_i - mu_i) / sigma_i (a standardised score does not fit the 16-bit
-// key of a bf16 coordinate). Each lane keeps its R best words; the k-th of the
+// Level 0 on 64-bit words of fp32 scores z(i) of the d coordinates (a
+// standardised score, or an fp32 coordinate, does not fit the 16-bit key of a
+// bf16 coordinate): the union path above. Each lane keeps its R best words;
+// the k-th of the
 // union is the threshold, and the few words at or above it that a lane did not
 // keep (found by rescanning only the lanes that can hold them) are merged in.
-// Returns false (nothing written) when they overflow E.
-template <int R, int KPL>
-__device__ __forceinline__ bool level0_union_std(const Args &a, const uint16_t *xh, int k, uint64_t *E, int ecap,
-                                                 uint64_t *L, uint32_t *beam) {
-    const int lane = threadIdx.x & 31, d = a.d;
+// Returns false (nothing written) when they overflow E. zq(i) is z(i) again,
+// for the rescan (without the status flag of a bad sigma).
+template <int R, int KPL, class Z, class Zq>
+__device__ __forceinline__ bool level0_union64(Z z, Zq zq, int d, int k, uint64_t *E, int ecap, uint64_t *L,
+                                               uint32_t *beam) {
+    const int lane = threadIdx.x & 31;
     uint64_t top[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) top[r] = 0ull;
 #pragma unroll 1
     for (int i = lane; i < d; i += 32) {
-        uint64_t c = cword(standardise(x_at(xh, i), (uint32_t)i, a, a.status), (uint32_t)i);
+        uint64_t c = cword(z(i), (uint32_t)i);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const uint64_t hi = whi(top[r], c);
@@ -592,7 +594,7 @@ __device__ __forceinline__ bool level0_union_std(const Args &a, const uint16_t *
             const int i = owner + 32 * j;
             const uint64_t km = __shfl_sync(kFull, kept_min, owner);
             uint64_t w = 0ull;
-            if (q < nf * ne && i < d) w = cword(standardise(x_at(xh, i), (uint32_t)i, a, nullptr), (uint32_t)i);
+            if (q < nf * ne && i < d) w = cword(zq(i), (uint32_t)i);
             const bool take = w >= tau && w < km && w != 0ull;
             const unsigned mb = __ballot_sync(kFull, take);
             const int pos = total + __popc(mb & lanes_below());
@@ -623,12 +625,13 @@ __device__ __forceinline__ bool level0_union_std(const Args &a, const uint16_t *
 // General path: every coordinate (standardised if tables are given) is a
 // candidate; a threshold that at least k of them reach keeps them in the
 // scratch (z, id) lists of capacity `cap`, the k-th is found by bisection, and
-// the first k, sorted, become the code list; its first 8 are the beam.
-template <bool STD>
-__device__ __forceinline__ void level0_bisect(const Args &a, const uint16_t *xh, float *pz, uint32_t *pid, int cap,
+// the first k, sorted, become the code list; its first 8 are the beam. zf(i)
+// is the score of coordinate i, zq(i) the same without the status flag, and
+// lowbit the lowest key bit that can be set.
+template <class Z, class Zq>
+__device__ __forceinline__ void level0_bisect(Z zf, Zq zq, int lowbit, int d, int k, float *pz, uint32_t *pid, int cap,
                                               uint64_t *L, uint32_t *beam) {
-    const int lane = threadIdx.x & 31, d = a.d, k = a.k;
-    const int lowbit = STD ? 0 : 16;  // keys of unstandardised bf16 values have 16 zero bits
+    const int lane = threadIdx.x & 31;
     // Each lane's R best keys, R = 2 ceil(k / 32) (at most 8): their union
     // holds at least k keys, and its k-th largest is a threshold that at least
     // k candidates reach and, unlike the smallest of the lanes' R-th keys,
@@ -638,7 +641,7 @@ __device__ __forceinline__ void level0_bisect(const Args &a, const uint16_t *xh,
 #pragma unroll
     for (int r = 0; r < 8; ++r) best[r] = 0u;
     for (int i = lane; i < d; i += 32) {
-        uint32_t kv = akey(stdz<STD>(x_at(xh, i), (uint32_t)i, a, a.status)) + 1u;
+        uint32_t kv = akey(zf(i)) + 1u;
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             if (r < R && kv > best[r]) {
@@ -663,7 +666,7 @@ __device__ __forceinline__ void level0_bisect(const Args &a, const uint16_t *xh,
         float z = 0.f;
         bool take = false;
         if (i < d) {
-            z = stdz<STD>(x_at(xh, i), (uint32_t)i, a, nullptr);
+            z = zq(i);
             take = akey(z) + 1u >= tau_low;
         }
         if (n + __popc(__ballot_sync(kFull, take)) > cap) {
@@ -681,14 +684,14 @@ __device__ __forceinline__ void level0_bisect(const Args &a, const uint16_t *xh,
             const uint32_t c = tau | (1u << b);
             int cnt = 0;
             for (int i = lane; i < d; i += 32)
-                cnt += akey(stdz<STD>(x_at(xh, i), (uint32_t)i, a, nullptr)) >= c;
+                cnt += akey(zq(i)) >= c;
             if (__reduce_add_sync(kFull, cnt) >= k) tau = c;
         }
         n = 0;
         for (int i0 = 0; i0 < d; i0 += 32) {
             const int i = i0 + lane;
             float z = 0.f;
-            if (i < d) z = stdz<STD>(x_at(xh, i), (uint32_t)i, a, nullptr);
+            if (i < d) z = zq(i);
             n = warp_append(pz, pid, n, i < d && akey(z) > tau, z, (uint32_t)i);
         }
         for (int i0 = 0; i0 < d && n < k; i0 += 32) {
@@ -696,7 +699,7 @@ __device__ __forceinline__ void level0_bisect(const Args &a, const uint16_t *xh,
             float z = 0.f;
             bool tie = false;
             if (i < d) {
-                z = stdz<STD>(x_at(xh, i), (uint32_t)i, a, nullptr);
+                z = zq(i);
                 tie = akey(z) == tau;
             }
             const unsigned mb = __ballot_sync(kFull, tie);
@@ -804,14 +807,17 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
             uint32_t *bt = beams + tk * kBeam;
             bool done = false;
             // each lane keeps R words, so the union of 32 R holds at least 2 k
+            const uint16_t *xt16 = xh + tk * nblk * 32;
+            auto zf = [&](int i) { return stdz<STD>(x_at(xt16, i), (uint32_t)i, a, a.status); };
+            auto zq = [&](int i) { return stdz<STD>(x_at(xt16, i), (uint32_t)i, a, nullptr); };
             if constexpr (KPL <= 4) {
                 if constexpr (STD)
-                    done = level0_union_std<(KPL <= 2 ? 4 : 8), KPL>(a, xh + tk * nblk * 32, k, E, a.ecap, Lt, bt);
+                    done = level0_union64<(KPL <= 2 ? 4 : 8), KPL>(zf, zq, d, k, E, a.ecap, Lt, bt);
                 else
                     done = level0_union<(KPL <= 2 ? 4 : 8), KPL>(row, nch, k, E, a.ecap, Lt, bt);
             }
-            if (!done)
-                level0_bisect<STD>(a, xh + tk * nblk * 32, reinterpret_cast<float *>(E),
+            if (!done)  // keys of unstandardised bf16 values have 16 zero bits
+                level0_bisect(zf, zq, STD ? 0 : 16, d, k, reinterpret_cast<float *>(E),
                               reinterpret_cast<uint32_t *>(E) + a.ecap, a.ecap, Lt, bt);
             if constexpr (WIDE) {  // the beam: the first 16 of the sorted list (k >= beam)
                 if (lane < 16) beams[lane] = cword_idx(Lt[lane]);

@@ -35,6 +35,11 @@ struct dpb_plan {
     bool mma_encode = false;
     std::vector<uint32_t> FRAG;
     std::vector<uint32_t> DD;
+    // FMA encoder tables (built when fma_encode is set; DD too): GF[l-1][q][w][lane][4],
+    // the generator signs +-1 of level l as fp32, generators 4 w .. 4 w + 3 at
+    // coordinate 32 q + lane (1 past d).
+    bool fma_encode = false;
+    std::vector<float> GF;
     // Per-level (tensor-core) encoder tables, built for DPB_SELECT_PER_LEVEL:
     //  GT: every level's generator signs gamma_j as bf16 +-1, per 64-coordinate
     //    chunk a [Delta_l][64] tile in the K-major core-matrix layout of
@@ -54,6 +59,7 @@ struct dpb_plan {
     uint32_t *dDD = nullptr;    // device copy of DD
     uint32_t *dGT = nullptr;    // device copy of GT
     uint32_t *dVH2 = nullptr;   // device copy of VH2
+    float *dGF = nullptr;       // device copy of GF
     // Coset-generator scoring (DPB_SCORING_COSET_WHT), per level l >= 1:
     //  COSET[(l-1) * (nblk + 16) + m] = sign word of g0 over 32-coordinate
     //  block m (bit i = parity(M[32 m + i] AND g0)), then 16 words S_j with
@@ -75,8 +81,10 @@ __host__ __device__ inline uint32_t dedup_hash(uint32_t delta) {
 // lane with q4 = lane % 4 the coordinates q4 + 4 j (j < 8), paired (j, j + 4).
 __host__ __device__ inline int frag_coord(int q4, int pair, int half) { return q4 + 4 * (pair + 4 * half); }
 
-// Builds the tensor-core encoder tables when the plan qualifies (dpb_plan.cu).
+// Builds the tensor-core encoder tables, or else the FMA encoder's, when the
+// plan qualifies (dpb_plan.cu).
 void build_mma_tables(dpb_plan *p);
+void build_fma_tables(dpb_plan *p);
 
 // Per-level encoder (dpb_encode_pl.cu): support check, tables, launch.
 dpb_status check_per_level(const dpb_config &c);
@@ -115,6 +123,8 @@ dpb_status resolve_and_build(const dpb_config *in, const uint32_t *generators, d
 cudaError_t launch_encode_mma(const dpb_plan *p, const void *x, int64_t T, const float *mu,
                               const float *sigma, const float2 *tab, int32_t *idx, float *val, float *xnorm,
                               int32_t *status, cudaStream_t stream);
+cudaError_t launch_encode_fma(const dpb_plan *p, const void *x, int64_t T, const float *mu, const float *sigma,
+                              int32_t *idx, float *val, float *xnorm, int32_t *status, cudaStream_t stream);
 // tab_scratch (nullable, tab_bytes(p) bytes): where the standardisation tables
 // are packed as (mu, 1 / sigma) pairs before the encoder runs.
 cudaError_t launch_encode(const dpb_plan *p, const void *x, int64_t T, const float *mu,

@@ -149,6 +149,28 @@ int ceil_log2(int v) {
 
 }  // namespace
 
+// The generator-difference tables DD of every level (children = 16).
+static void build_dedup(dpb_plan *p) {
+    const dpb_config &c = p->cfg;
+    p->DD.assign((size_t)(c.levels - 1) * kDedupSlots, 0u);
+    for (int l = 1; l < c.levels; ++l) {
+        uint32_t *tab = &p->DD[(size_t)(l - 1) * kDedupSlots];
+        const uint32_t *g = &p->G[(size_t)l * DPB_MAX_CHILDREN];
+        // parents of level l lie below 2^bits[l-1], so only differences below
+        // that bound can make two parents share a child
+        const uint32_t bound = 1u << c.bits[l - 1];
+        for (int j = 0; j < 16; ++j)
+            for (int jj = 0; jj < 16; ++jj) {
+                if (j == jj) continue;
+                const uint32_t delta = g[j] ^ g[jj];
+                if (delta >= bound) continue;
+                uint32_t h = dedup_hash(delta);
+                while (tab[h] != 0) h = (h + 1) & (kDedupSlots - 1);
+                tab[h] = ((delta + 1) << 4) | (uint32_t)j;
+            }
+    }
+}
+
 void build_mma_tables(dpb_plan *p) {
     const dpb_config &c = p->cfg;
     bool ok = c.dtype == DPB_BF16 && c.d % 32 == 0 && c.d >= 32 && c.d <= 1024 && c.levels >= 2 &&
@@ -178,23 +200,24 @@ void build_mma_tables(dpb_plan *p) {
                     p->FRAG[((((size_t)(l - 1) * nblk + m) * 2 + chunk) * 32 + lane) * 4 + w % 4] =
                         sign_bf16(g, ia) | (sign_bf16(g, ib) << 16);
                 }
-    p->DD.assign((size_t)(c.levels - 1) * kDedupSlots, 0u);
-    for (int l = 1; l < c.levels; ++l) {
-        uint32_t *tab = &p->DD[(size_t)(l - 1) * kDedupSlots];
-        const uint32_t *g = &p->G[(size_t)l * DPB_MAX_CHILDREN];
-        // parents of level l lie below 2^bits[l-1], so only differences below
-        // that bound can make two parents share a child
-        const uint32_t bound = 1u << c.bits[l - 1];
-        for (int j = 0; j < 16; ++j)
-            for (int jj = 0; jj < 16; ++jj) {
-                if (j == jj) continue;
-                const uint32_t delta = g[j] ^ g[jj];
-                if (delta >= bound) continue;
-                uint32_t h = dedup_hash(delta);
-                while (tab[h] != 0) h = (h + 1) & (kDedupSlots - 1);
-                tab[h] = ((delta + 1) << 4) | (uint32_t)j;
-            }
-    }
+    build_dedup(p);
+}
+
+void build_fma_tables(dpb_plan *p) {
+    const dpb_config &c = p->cfg;
+    bool ok = !p->mma_encode && c.levels >= 2 && c.select_mode == DPB_SELECT_GLOBAL && c.beam <= 16 && c.k >= c.beam &&
+              c.bits[c.levels - 2] <= 27;
+    for (int l = 1; l < c.levels && ok; ++l) ok = c.children[l] == 16;
+    p->fma_encode = ok;
+    if (!ok) return;
+    const int nq = (c.d + 31) / 32;
+    p->GF.assign((size_t)(c.levels - 1) * nq * 512, 1.f);
+    for (int l = 1; l < c.levels; ++l)
+        for (int i = 0; i < c.d; ++i)
+            for (int j = 0; j < 16; ++j)
+                if (__builtin_popcount(p->M[i] & p->G[(size_t)l * DPB_MAX_CHILDREN + j]) & 1)
+                    p->GF[((((size_t)(l - 1) * nq + i / 32) * 4 + j / 4) * 32 + i % 32) * 4 + j % 4] = -1.f;
+    build_dedup(p);
 }
 
 dpb_status fail(dpb_status s, const char *fmt, ...) {
@@ -336,6 +359,7 @@ dpb_status resolve_and_build(const dpb_config *in, const uint32_t *generators, d
     }
     p->cfg = c;
     build_mma_tables(p);
+    build_fma_tables(p);
     if (c.scoring == DPB_SCORING_COSET_WHT) {
         // the variant outside the paper: every level's 16 generators one coset
         // g0 ^ {0..15} (given by the caller), scored by a 16-point WHT
