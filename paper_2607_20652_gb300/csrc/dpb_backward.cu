@@ -304,7 +304,7 @@ __device__ __forceinline__ void analyse(const BwdWarp &w, int nh, int d, const u
 // KEPT: norm matching with the decode's r given (a separate instantiation,
 // without the path that rebuilds r).
 template <typename Tio, int NKC, bool VEC, bool KEPT>
-__global__ void __launch_bounds__(kBwdWarps * 32, 2) backward_lut_kernel(BackwardArgs a, int t) {
+__global__ void __launch_bounds__(kBwdWarps * 32, 2) backward_lut_kernel(BackwardArgs a, int t, bool spread) {
     extern __shared__ __align__(16) uint32_t smem_raw[];
     uint32_t *smem = aligned_smem<256>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -337,7 +337,8 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2) backward_lut_kernel(Backwar
     const Tio *X = static_cast<const Tio *>(a.x);
     const Tio *GY = static_cast<const Tio *>(a.gy);
     Tio *GX = static_cast<Tio *>(a.gx);
-    for (int64_t tk = (int64_t)blockIdx.x * nwarps + warp; tk < a.T; tk += (int64_t)gridDim.x * nwarps) {
+    for (int64_t tk = spread ? (int64_t)warp * gridDim.x + blockIdx.x : (int64_t)blockIdx.x * nwarps + warp;
+         tk < a.T; tk += (int64_t)gridDim.x * nwarps) {
         const int32_t *it = a.idx + tk * k;
         const float *vt = a.val + tk * k;
         const Tio *xr = X + tk * d, *gr = GY + tk * d;
@@ -478,21 +479,20 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2) backward_lut_kernel(Backwar
     }
 }
 
-int grid_for(const dpb_plan *p, int64_t T, int warps) {
-    return (int)std::min<int64_t>((T + warps - 1) / warps, (int64_t)std::max(p->sms, 1) * 16);
-}
-
 template <typename Tio, int NKC, bool VEC, bool KEPT>
 cudaError_t run_backward_lut(const dpb_plan *p, const BackwardArgs &a, int64_t T, cudaStream_t stream) {
     const size_t per_block = 256 /* alignment */ + sizeof(uint32_t) * (size_t)bwd_block_words(p->cfg.d, NKC);
     const size_t per_warp = sizeof(uint32_t) * (size_t)bwd_warp_words(p->cfg.d, p->code_len, NKC);
     const void *fn = (const void *)backward_lut_kernel<Tio, NKC, VEC, KEPT>;
-    const int warps = best_warps(fn, kBwdWarps, per_block, per_warp);
+    const Fit fit = best_warps(fn, kBwdWarps, per_block, per_warp);
+    const int warps = fit.warps;
     if (warps <= 0) return cudaErrorInvalidConfiguration;
+    bool spread;
+    const int grid = grid_for(p, T, fit, spread);
     const size_t smem = per_block + (size_t)warps * per_warp;
     const cudaError_t e = allow_smem((const void *)backward_lut_kernel<Tio, NKC, VEC, KEPT>, smem);
     if (e != cudaSuccess) return e;
-    backward_lut_kernel<Tio, NKC, VEC, KEPT><<<grid_for(p, T, warps), warps * 32, smem, stream>>>(a, p->t);
+    backward_lut_kernel<Tio, NKC, VEC, KEPT><<<grid, warps * 32, smem, stream>>>(a, p->t, spread);
     return cudaGetLastError();
 }
 
@@ -543,7 +543,7 @@ cudaError_t launch_backward(const dpb_plan *p, const void *x, const int32_t *idx
     int warps = 4;
     while (warps > 1 && sizeof(uint32_t) * ((size_t)c.d + (size_t)warps * 4 * c.d) > kMaxSmemPerBlock) --warps;
     const size_t smem = sizeof(uint32_t) * ((size_t)c.d + (size_t)warps * 4 * c.d);
-    const int grid = grid_for(p, T, warps);
+    const int grid = (int)std::min<int64_t>((T + warps - 1) / warps, (int64_t)std::max(p->sms, 1) * 16);
     if (c.dtype == DPB_BF16) {
         const cudaError_t e = allow_smem((const void *)backward_warp_kernel<__nv_bfloat16>, smem);
         if (e != cudaSuccess) return e;

@@ -32,18 +32,18 @@ cudaError_t allow_smem(const void *func, size_t bytes) {
     return e;
 }
 
-int best_warps(const void *func, int max_warps, size_t per_block, size_t per_warp) {
+Fit best_warps(const void *func, int max_warps, size_t per_block, size_t per_warp) {
     static std::mutex mu;
-    static std::map<std::tuple<const void *, int, size_t, size_t>, int> chosen;
+    static std::map<std::tuple<const void *, int, size_t, size_t>, Fit> chosen;
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return Fit{};
     const auto key = std::make_tuple(func, dev, per_block, per_warp);
     {
         std::lock_guard<std::mutex> lock(mu);
         const auto it = chosen.find(key);
         if (it != chosen.end()) return it->second;
     }
-    int best = 0, best_resident = 0;
+    Fit best;
     for (int w = max_warps; w >= 1; --w) {
         const size_t smem = per_block + (size_t)w * per_warp;
         if (smem > kMaxSmemPerBlock || allow_smem(func, smem) != cudaSuccess) continue;
@@ -52,10 +52,7 @@ int best_warps(const void *func, int max_warps, size_t per_block, size_t per_war
             cudaGetLastError();
             continue;
         }
-        if (blocks * w > best_resident) {
-            best_resident = blocks * w;
-            best = w;
-        }
+        if (blocks * w > best.blocks * best.warps) best = Fit{w, blocks};
     }
     std::lock_guard<std::mutex> lock(mu);
     chosen[key] = best;

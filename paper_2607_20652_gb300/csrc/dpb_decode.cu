@@ -122,7 +122,7 @@ __device__ __forceinline__ float keep_r(float *R, const float *r, int d) {
 
 // KEPT: norm matching, and r kept for the backward (a separate instantiation).
 template <typename Tio, int NKC, bool VEC, bool KEPT>
-__global__ void __launch_bounds__(kDecWarps * 32, 4) decode_lut_kernel(DecodeArgs a, int t) {
+__global__ void __launch_bounds__(kDecWarps * 32, 4) decode_lut_kernel(DecodeArgs a, int t, bool spread) {
     extern __shared__ __align__(16) uint32_t smem_raw[];
     uint32_t *smem = aligned_smem<128>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -136,7 +136,8 @@ __global__ void __launch_bounds__(kDecWarps * 32, 4) decode_lut_kernel(DecodeArg
     float *r = reinterpret_cast<float *>(base + sww);
     HashedList hl{base + sww + dp, reinterpret_cast<float *>(base + sww + dp + kp), nullptr};
     Tio *Y = static_cast<Tio *>(a.y);
-    for (int64_t tk = (int64_t)blockIdx.x * nwarps + warp; tk < a.T; tk += (int64_t)gridDim.x * nwarps) {
+    for (int64_t tk = spread ? (int64_t)warp * gridDim.x + blockIdx.x : (int64_t)blockIdx.x * nwarps + warp;
+         tk < a.T; tk += (int64_t)gridDim.x * nwarps) {
         RowOps<VEC>::fill(r, d, 0.f);
         __syncwarp();
         const int nh = split_code(a.idx + tk * a.k, a.val + tk * a.k, a.k, d, a.m_mask, r, hl, a.status);
@@ -159,10 +160,6 @@ __global__ void __launch_bounds__(kDecWarps * 32, 4) decode_lut_kernel(DecodeArg
     }
 }
 
-int grid_for(const dpb_plan *p, int64_t T, int warps) {
-    return (int)std::min<int64_t>((T + warps - 1) / warps, (int64_t)std::max(p->sms, 1) * 16);
-}
-
 }  // namespace
 
 namespace {
@@ -172,12 +169,15 @@ cudaError_t run_decode_lut(const dpb_plan *p, const DecodeArgs &a, int64_t T, cu
     const size_t per_block = 128 /* alignment */ + sizeof(uint32_t) * (size_t)pad32(p->cfg.d);
     const size_t per_warp = sizeof(uint32_t) * (size_t)decode_warp_words(p->cfg.d, p->code_len, NKC);
     const void *fn = (const void *)decode_lut_kernel<Tio, NKC, VEC, KEPT>;
-    const int warps = best_warps(fn, kDecWarps, per_block, per_warp);
+    const Fit fit = best_warps(fn, kDecWarps, per_block, per_warp);
+    const int warps = fit.warps;
     if (warps <= 0) return cudaErrorInvalidConfiguration;
+    bool spread;
+    const int grid = grid_for(p, T, fit, spread);
     const size_t smem = per_block + (size_t)warps * per_warp;
     const cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
-    decode_lut_kernel<Tio, NKC, VEC, KEPT><<<grid_for(p, T, warps), warps * 32, smem, stream>>>(a, p->t);
+    decode_lut_kernel<Tio, NKC, VEC, KEPT><<<grid, warps * 32, smem, stream>>>(a, p->t, spread);
     return cudaGetLastError();
 }
 
@@ -218,7 +218,7 @@ cudaError_t launch_decode(const dpb_plan *p, const int32_t *idx, const float *va
     int warps = 4;  // fewer when the two d-length buffers per warp would not fit
     while (warps > 1 && sizeof(uint32_t) * ((size_t)c.d + (size_t)warps * 2 * c.d) > kMaxSmemPerBlock) --warps;
     const size_t smem = sizeof(uint32_t) * ((size_t)c.d + (size_t)warps * 2 * c.d);
-    const int grid = grid_for(p, T, warps);
+    const int grid = (int)std::min<int64_t>((T + warps - 1) / warps, (int64_t)std::max(p->sms, 1) * 16);
     if (c.dtype == DPB_BF16) {
         const cudaError_t e = allow_smem((const void *)decode_warp_kernel<__nv_bfloat16>, smem);
         if (e != cudaSuccess) return e;

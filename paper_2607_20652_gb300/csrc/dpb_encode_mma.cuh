@@ -64,8 +64,9 @@ struct Args {
 // ---- shared-memory layout (32-bit words) ------------------------------------------
 
 __host__ __device__ inline int block_words(int levels, int nblk, int nkc) {
-    // frag [(L-1)][nblk][2][32][4], W5 [32], VH [nkc][32][32], DD [(L-1)][kDedupSlots], G [L][16]
-    return (levels - 1) * nblk * 256 + 32 + nkc * 1024 + (levels - 1) * kDedupSlots + 8 * 16;
+    // frag [(L-1)][nblk][2][32][4], W5 [32], VH [nkc][32][32], DD [(L-1)][kDedupSlots], G [L][16],
+    // the tables' mbarrier (2, padded to 4)
+    return (levels - 1) * nblk * 256 + 32 + nkc * 1024 + (levels - 1) * kDedupSlots + 8 * 16 + 4;
 }
 
 // 64-bit entries of the per-warp scratch buffer: the entrants of a merge, the
@@ -112,6 +113,29 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
         "{%0,%1,%2,%3};\n"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) into
+// shared memory, completing on the mbarrier at `bar`.
+__device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+
+// Waits (at most 2^20 polls) for the first phase of the mbarrier at `bar`.
+__device__ __forceinline__ bool tables_landed(uint32_t bar) {
+    for (int i = 0; i < 1 << 20; ++i) {
+        uint32_t done;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(bar)
+            : "memory");
+        if (done) return true;
+    }
+    return false;
 }
 
 // Parts of parent p's sign words: its Walsh word, the block-parity word
@@ -748,24 +772,30 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
     uint32_t *s_vh = s_w5 + 32;
     uint32_t *s_dd = s_vh + NKC * 1024;
     uint32_t *s_g = s_dd + (L - 1) * kDedupSlots;
-    {
-        if (COSET) {
-            for (int i = threadIdx.x; i < (L - 1) * (nblk + 16); i += blockDim.x) s_frag[i] = a.coset[i];
-        } else {
-            const uint4 *src = reinterpret_cast<const uint4 *>(a.frag);
-            uint4 *dst = reinterpret_cast<uint4 *>(s_frag);
-            for (int i = threadIdx.x; i < (L - 1) * nblk * 64; i += blockDim.x) dst[i] = src[i];
-        }
-        for (int v = threadIdx.x; v < 32; v += blockDim.x) {
-            uint32_t word = 0;
-            for (int l = 0; l < 32; ++l) word |= (uint32_t)(__popc(l & v) & 1) << l;
-            s_w5[v] = word;
-        }
-        for (int i = threadIdx.x; i < NKC * 1024; i += blockDim.x) s_vh[i] = a.VH[i];
-        for (int i = threadIdx.x; i < (L - 1) * kDedupSlots; i += blockDim.x) s_dd[i] = a.DD[i];
-        for (int i = threadIdx.x; i < L * 16; i += blockDim.x) s_g[i] = a.G[(i >> 4) * DPB_MAX_CHILDREN + (i & 15)];
+    uint32_t *s_bar = s_g + 8 * 16;
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(s_bar);
+    if (threadIdx.x == 0) {
+        // the large tables by bulk copies that land while level 0, which reads none of them, runs
+        const uint32_t nf = COSET ? 0u : (uint32_t)(L - 1) * nblk * 1024u, nv = NKC * 4096u;
+        const uint32_t nd = (uint32_t)(L - 1) * kDedupSlots * 4u;
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+        asm volatile("fence.mbarrier_init.release.cluster;");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(nf + nv + nd)
+                     : "memory");
+        if (!COSET) bulk_copy(s_frag, a.frag, nf, bar);
+        bulk_copy(s_vh, a.VH, nv, bar);
+        bulk_copy(s_dd, a.DD, nd, bar);
     }
+    if (COSET)
+        for (int i = threadIdx.x; i < (L - 1) * (nblk + 16); i += blockDim.x) s_frag[i] = a.coset[i];
+    for (int v = threadIdx.x; v < 32; v += blockDim.x) {
+        uint32_t word = 0;
+        for (int l = 0; l < 32; ++l) word |= (uint32_t)(__popc(l & v) & 1) << l;
+        s_w5[v] = word;
+    }
+    for (int i = threadIdx.x; i < L * 16; i += blockDim.x) s_g[i] = a.G[(i >> 4) * DPB_MAX_CHILDREN + (i & 15)];
     __syncthreads();
+    bool tables = false;  // the copies are seen to have landed
 
     uint32_t *xt = smem + block_words(L, nblk, NKC) + warp * warp_words(nblk, k);
     uint64_t *codes = reinterpret_cast<uint64_t *>(xt + 2 * nblk * 16);  // [2][k]
@@ -777,11 +807,16 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
     // the lane-th slot pair (sp, s), sp < s, of the beam
     const int ps = 1 + (lane >= 1) + (lane >= 3) + (lane >= 6) + (lane >= 10) + (lane >= 15) + (lane >= 21);
     const int psp = lane - ps * (ps - 1) / 2;
-    const int64_t npairs = WIDE ? a.T : (a.T + 1) / 2;
-
-    for (int64_t pr = (int64_t)blockIdx.x * nwarps + warp; pr < npairs; pr += (int64_t)gridDim.x * nwarps) {
-        const int64_t t0 = WIDE ? pr : 2 * pr;
-        const int ntok = WIDE ? 1 : (t0 + 1 < a.T ? 2 : 1);
+    // Warps are numbered across the blocks (block b's warp w is w gridDim.x + b),
+    // so that every SM gets the same share of a batch of any size. A round gives
+    // each warp two tokens (WIDE: one); the last round's tokens go one to a
+    // warp, and a second one only to as many warps as it takes.
+    const int64_t W = (int64_t)gridDim.x * nwarps, gw = (int64_t)warp * gridDim.x + blockIdx.x;
+    for (int64_t base = 0; base < a.T; base += WIDE ? W : 2 * W) {
+        const int64_t two = WIDE ? 0 : min(max(a.T - base - W, (int64_t)0), W);  // warps with two tokens
+        const int64_t t0 = base + (gw < two ? 2 * gw : two + gw);
+        const int ntok = gw < two ? 2 : 1;
+        if (t0 >= a.T) break;
         const int nhalf = WIDE ? 2 : ntok;  // row groups of 8 beam slots
 
         // ---- each row into the permuted tile; |x|; level 0 ----
@@ -825,6 +860,13 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
             }
         }
 
+        if (!tables) {
+            if (!tables_landed(bar)) {  // never seen: the copies are the block's own
+                set_status(a.status, DPB_DEV_TIMEOUT);
+                return;
+            }
+            tables = true;
+        }
         // ---- levels 1 .. L-1 ----
         for (int l = 1; l < L; ++l) {
             const uint32_t *frag = s_frag + (l - 1) * nblk * 256;
@@ -930,7 +972,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
                 for (int tk = 0; tk < 2; ++tk)
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
-                        if (tk < nhalf)
+                        if (tk < nhalf && (WIDE ? 8 * tk : 0) + slot < a.beam)  // slots that hold a parent
                             sc[tk][e] = standardise(sc[tk][e], (tk ? p1 : p0) ^ gl[8 * (e >> 1) + 2 * q4 + (e & 1)],
                                                     a, a.status);
             }
@@ -1066,8 +1108,7 @@ cudaError_t launch_kpl_std(const dpb_plan *p, const Args &a, int warps, cudaStre
     const size_t smem = encode_mma_smem(p, warps);
     const cudaError_t e = allow_smem((const void *)encode_kernel<NKC, KPL, COSET, WIDE, STD>, smem);
     if (e != cudaSuccess) return e;
-    const int64_t pairs = WIDE ? a.T : (a.T + 1) / 2;
-    const int grid = (int)std::min<int64_t>((pairs + warps - 1) / warps, (int64_t)std::max(p->sms, 1));
+    const int grid = (int)std::min<int64_t>(a.T, (int64_t)std::max(p->sms, 1));
     encode_kernel<NKC, KPL, COSET, WIDE, STD><<<grid, warps * 32, smem, stream>>>(a);
     return cudaGetLastError();
 }

@@ -58,3 +58,27 @@ def test_fma_encoder_groups_of_rows_are_independent():
     for n in (1, 2, 3):
         i, v, q = dpb.encode(plan, x[:n].contiguous())
         assert torch.equal(i, idx[:n]) and torch.equal(v, val[:n]) and torch.equal(q, xn[:n])
+
+
+@pytest.mark.parametrize("beam,k,std", [(8, 64, False), (16, 32, False), (4, 5, True)])
+def test_rows_do_not_depend_on_their_batch(beam, k, std):
+    """Every share of tokens among the warps (a token or two to a warp, full and
+    partial rounds, spread and blockwise grids) gives a row the same bits."""
+    plan = dpb.Plan(d=96, levels=4, m_bits=14, children=16, beam=beam, k=k, dtype="bf16")
+    mu = sigma = None
+    if std:
+        mu, sigma = (torch.from_numpy(t).cuda() for t in inputs.moment_tables(plan.n_features, 5))
+    base = torch.from_numpy(inputs.gaussian_rows(64, 96, 3)).cuda().to(torch.bfloat16)
+    gyb = torch.from_numpy(inputs.normal((64, 96), 4)).cuda().to(torch.bfloat16)
+    want = None
+    for T in (64, 1, 151, 153, 1375, 3041, 4577, 6081, 9001, 12321):
+        rows = torch.arange(T, device="cuda") % 64
+        x, gy = base[rows].contiguous(), gyb[rows].contiguous()
+        r = torch.empty((T, 96), dtype=torch.float32, device="cuda")
+        code = dpb.forward(plan, x, mu, sigma, r_out=r)
+        out = code + (r,) + dpb.backward(plan, x, code[0], code[1], gy, sigma=sigma, r=r)
+        if want is None:
+            want = out
+        for w, o in zip(want, out):
+            assert torch.equal(w[rows], o), T
+    assert plan.status() == 0
