@@ -448,17 +448,14 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2) backward_lut_kernel(Backwar
                     a.gval[tk * k + e] = gvv;
                 }
                 __syncwarp();
-                // ---- grad_x: direct term and basis terms, then the hashed sum ----
-                const float dx = nx > 0.f ? direct / nx : 0.f;
-                RowOps<VEC>::scale_in(w.buf, xr, d, dx);
-                __syncwarp();
-                for (int e = lane; e < k; e += 32) {
-                    const int cm = w.cmap[e];
-                    if (cm < 0 && cm != INT_MIN) w.buf[-cm - 1] += bterm[e];  // indices are distinct
-                }
-                __syncwarp();
             }
-            synthesise<NKC, kSweepCompact>(sw, w.hc, w.ha, nh, t, d, koff, a.inv_sqrt_d, w.buf);
+            // pass 0 adds to the basis part of r in buf; pass 1 writes the hashed
+            // part of grad_x over dL/dr, which nothing reads any more
+            if (nh > 0)
+                synthesise<NKC, false>(sw, w.hc, w.ha, nh, t, d, koff, a.inv_sqrt_d, w.buf, pass == 0);
+            else if (pass == 1)
+                RowOps<VEC>::fill(w.buf, d, 0.f);
+            __syncwarp();
             if (pass == 1) break;
             // ---- dL/dr = c (g - (<g,r>/|r|^2) r) in place of r ----
             float srr = 0.f, sgr = 0.f;
@@ -474,7 +471,13 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2) backward_lut_kernel(Backwar
             }
             __syncwarp();
         }
-        RowOps<VEC>::store(GX + tk * d, w.buf, d, 1.f);
+        // ---- grad_x: the basis terms onto the hashed part, then the direct term ----
+        for (int e = lane; e < k; e += 32) {
+            const int cm = w.cmap[e];
+            if (cm < 0 && cm != INT_MIN) w.buf[-cm - 1] += bterm[e];  // indices are distinct
+        }
+        __syncwarp();
+        RowOps<VEC>::store_axpy(GX + tk * d, w.buf, xr, d, nx > 0.f ? direct / nx : 0.f);
         __syncwarp();
     }
 }

@@ -149,9 +149,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, 4) decode_lut_kernel(DecodeArg
         } else {
             if (a.R) RowOps<VEC>::store(a.R + tk * d, r, d, 1.f);
             if (a.norm_match) {
-                float ss = 0.f, unused = 0.f;
-                RowOps<VEC>::dots(r, r, d, ss, unused);
-                const float nr = sqrtf(warp_sum(ss));
+                const float nr = sqrtf(warp_sum(RowOps<VEC>::sumsq(static_cast<const float *>(r), d)));
                 scale = nr > 0.f ? a.xnorm[tk] / nr : 0.f;
             }
         }

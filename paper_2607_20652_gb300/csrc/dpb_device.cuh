@@ -149,6 +149,20 @@ struct RowOps {
             for (int i = lane; i < d; i += 32) buf[i] = c * (ld_elem(row, i) - beta * buf[i]);
         }
     }
+    // row[i] = buf[i] + c x[i]
+    template <typename T>
+    __device__ __forceinline__ static void store_axpy(T *row, const float *buf, const T *x, int d, float c) {
+        const int lane = threadIdx.x & 31;
+        if (VEC) {
+#pragma unroll 2
+            for (int i = 4 * lane; i < d; i += 128) {
+                const float4 r = *reinterpret_cast<const float4 *>(buf + i), v = ld4(x + i);
+                st4(row + i, make_float4(fmaf(c, v.x, r.x), fmaf(c, v.y, r.y), fmaf(c, v.z, r.z), fmaf(c, v.w, r.w)));
+            }
+        } else {
+            for (int i = lane; i < d; i += 32) st_elem(row, i, fmaf(c, ld_elem(x, i), buf[i]));
+        }
+    }
     // row[i] = c * buf[i]
     template <typename T>
     __device__ __forceinline__ static void store(T *row, const float *buf, int d, float c) {

@@ -39,13 +39,14 @@ constexpr int kMaxBlocks = 64;   // 32-coordinate blocks of d <= 2048
 // bytes), ZH (nkc tables of 2 x 32 words), the odd runs' value tables (6 x 32
 // words, 128-byte aligned) and the coefficients (64). A multiple of 32 words.
 __host__ __device__ constexpr int sweep_words(int qn, int nkc) {
-    return ((2 * qn + 31) & ~31) + 64 * nkc + 32 * (kMaxRuns - kShflRuns) + 64;
+    return ((qn + 1 + 31) & ~31) + 64 * nkc + 32 * (kMaxRuns - kShflRuns) + 64;
 }
 
 struct Sweep {
     uint2 zl;                 // ZL(lane) for codes 0..31 (x) and 32..63 (y)
+    uint2 zl1;                // ZL(lane) ^ ZQ(1): the odd block of a pair
     float vt[kShflRuns];      // lane v holds the table of run 2i at v
-    uint2 *zq;                // [qn] (shared)
+    uint2 *zq;                // [(qn + 1) / 2] of the even blocks (shared)
     uint32_t *zh;             // [nkc][2][32]: codes 0..31, then 32..63 (shared)
     float *vto;               // [6][32] odd runs (shared)
     float *coef;              // [64] (shared)
@@ -83,7 +84,7 @@ __device__ __forceinline__ uint32_t *aligned_smem(uint32_t *raw) {
 __device__ __forceinline__ Sweep sweep_at(uint32_t *base, int qn, int nkc) {
     Sweep s;
     s.zq = reinterpret_cast<uint2 *>(base);
-    s.zh = base + ((2 * qn + 31) & ~31);
+    s.zh = base + ((qn + 1 + 31) & ~31);
     s.vto = reinterpret_cast<float *>(s.zh + 64 * nkc);
     s.coef = s.vto + 32 * (kMaxRuns - kShflRuns);
     s.vto_s = smem_u32(s.vto);
@@ -120,15 +121,16 @@ __device__ __forceinline__ void sweep_build_signs(uint32_t ca, uint32_t cb, int 
         qa[b] = live ? __ballot_sync(kFull, (ca >> (5 + b)) & 1u) : 0u;
         qb[b] = live ? __ballot_sync(kFull, (cb >> (5 + b)) & 1u) : 0u;
     }
-    for (int q = lane; q < qn; q += 32) {
+    s.zl1 = make_uint2(zl.x ^ qa[0], zl.y ^ qb[0]);
+    for (int q = 2 * lane; q < qn; q += 64) {
         uint2 z = make_uint2(0u, 0u);
 #pragma unroll
-        for (int b = 0; b < 6; ++b)
+        for (int b = 1; b < 6; ++b)
             if ((q >> b) & 1) {
                 z.x ^= qa[b];
                 z.y ^= qb[b];
             }
-        s.zq[q] = z;
+        s.zq[q / 2] = z;
     }
 #pragma unroll
     for (int k = 0; k < kMaxKChunks; ++k) {
@@ -172,13 +174,14 @@ __device__ __forceinline__ void sweep_build_values(Sweep &s) {
     }
 }
 
-// Z(iota) of a sweep; koff = kappa_offsets4(inv iota), zq = ZQ(iota >> 5).
+// Z(iota) of a sweep; koff = kappa_offsets4(inv iota), zl = ZL(lane) (zl1 for
+// an odd block), zq = ZQ of the block's pair.
 // Each half of a ZH entry is its own 32-word table, so that a lookup of
 // random entries by the 32 lanes is free of bank conflicts.
 template <int NKC>
-__device__ __forceinline__ uint2 sweep_signs(const Sweep &s, uint2 zq, uint32_t koff) {
+__device__ __forceinline__ uint2 sweep_signs(const Sweep &s, uint2 zl, uint2 zq, uint32_t koff) {
     const char *zh = reinterpret_cast<const char *>(s.zh);
-    uint2 z = make_uint2(s.zl.x ^ zq.x, s.zl.y ^ zq.y);
+    uint2 z = make_uint2(zl.x ^ zq.x, zl.y ^ zq.y);
 #pragma unroll
     for (int k = 0; k < NKC; ++k) {
         const uint32_t o = __byte_perm(koff, 0, 0x4440 + k);
@@ -310,59 +313,66 @@ __device__ __forceinline__ int split_code(const int32_t *idx, const float *val, 
 
 // ---- synthesis over a hashed list ---------------------------------------------
 
-// out[i] += scale * sum over one sweep, for every coordinate of the token.
-// UNROLL coordinates blocks per loop trip.
-template <int NKC, int RUNS, int UNROLL>
+// out[i] += scale * sum over one sweep (= when ADD is not set and `add` is
+// false), for every coordinate of the token. Two 32-coordinate blocks per loop
+// trip: their ZQ words differ by a register constant, so one load serves both,
+// and their lookups are in flight together (one block per trip took the
+// backward of 65,536 tokens, d = 768, k = 64, 402 us, two 395).
+template <int NKC, int RUNS, bool ADD>
 __device__ __forceinline__ void sweep_accumulate(const Sweep &s, float *out, const uint32_t *koff, int d,
-                                                 float scale) {
+                                                 float scale, bool add) {
     const int lane = threadIdx.x & 31;
     const int qn = (d + 31) / 32;
-#pragma unroll UNROLL
-    for (int q = 0; q < qn; ++q) {
-        const int i = 32 * q + lane;
-        const bool in = i < d;
-        const uint2 z = sweep_signs<NKC>(s, s.zq[q], in ? koff[i] : 0u);
-        const float v = sweep_sum<RUNS>(s, z);
-        if (in) out[i] += scale * v;
+#pragma unroll 1
+    for (int q = 0; q < qn; q += 2) {
+        const int i = 32 * q + lane, j = i + 32;
+        const bool ii = i < d, jj = j < d;
+        const uint2 zq = s.zq[q >> 1];
+        const uint2 za = sweep_signs<NKC>(s, s.zl, zq, ii ? koff[i] : 0u);
+        const uint2 zb = sweep_signs<NKC>(s, s.zl1, zq, jj ? koff[j] : 0u);
+        if constexpr (ADD) {
+            const float va = sweep_sum<RUNS>(s, za);
+            if (ii) out[i] += scale * va;
+            const float vb = sweep_sum<RUNS>(s, zb);
+            if (jj) out[j] += scale * vb;
+        } else {
+            float va = scale * sweep_sum<RUNS>(s, za), vb = scale * sweep_sum<RUNS>(s, zb);
+            if (add) {
+                va += ii ? out[i] : 0.f;
+                vb += jj ? out[j] : 0.f;
+            }
+            if (ii) out[i] = va;
+            if (jj) out[j] = vb;
+        }
     }
 }
 
-// Code shape of a sweep. kSweepWide rounds the runs up to one of five
-// unrolled widths (the extra runs read all-zero tables) and does two blocks
-// per trip: the fewest instructions. kSweepCompact does one block per trip
-// and rounds the runs up to 8, 10 or 13 only: less code, for kernels whose
-// other phases already fill the instruction caches.
-enum SweepShape { kSweepWide, kSweepCompact };
-
-template <int NKC, SweepShape SHAPE>
+// The runs are rounded up to one of five unrolled widths (the extra runs read
+// all-zero tables). The narrow ones matter for the backward too: at k = 128 a
+// code's second sweep often has 3 runs (sweep point 2^22, beam 16: step 1,163 us
+// with 8, 10 and 13 only, 1,151 with 4 and 6 as well).
+template <int NKC, bool ADD>
 __device__ __forceinline__ void sweep_accumulate_runs(const Sweep &s, float *out, const uint32_t *koff,
-                                                      int d, float scale) {
-    if constexpr (SHAPE == kSweepCompact) {
-        if (s.runs <= 8)
-            sweep_accumulate<NKC, 8, 1>(s, out, koff, d, scale);
-        else if (s.runs <= 10)
-            sweep_accumulate<NKC, 10, 1>(s, out, koff, d, scale);
-        else
-            sweep_accumulate<NKC, kMaxRuns, 1>(s, out, koff, d, scale);
-    } else if (s.runs <= 4) {
-        sweep_accumulate<NKC, 4, 2>(s, out, koff, d, scale);
-    } else if (s.runs <= 6) {
-        sweep_accumulate<NKC, 6, 2>(s, out, koff, d, scale);
-    } else if (s.runs <= 8) {
-        sweep_accumulate<NKC, 8, 2>(s, out, koff, d, scale);
-    } else if (s.runs <= 10) {
-        sweep_accumulate<NKC, 10, 2>(s, out, koff, d, scale);
-    } else {
-        sweep_accumulate<NKC, kMaxRuns, 2>(s, out, koff, d, scale);
-    }
+                                                      int d, float scale, bool add) {
+    if (s.runs <= 4)
+        sweep_accumulate<NKC, 4, ADD>(s, out, koff, d, scale, add);
+    else if (s.runs <= 6)
+        sweep_accumulate<NKC, 6, ADD>(s, out, koff, d, scale, add);
+    else if (s.runs <= 8)
+        sweep_accumulate<NKC, 8, ADD>(s, out, koff, d, scale, add);
+    else if (s.runs <= 10)
+        sweep_accumulate<NKC, 10, ADD>(s, out, koff, d, scale, add);
+    else
+        sweep_accumulate<NKC, kMaxRuns, ADD>(s, out, koff, d, scale, add);
 }
 
 // out[i] += scale * sum_e coef_e (-1)^{parity(M[i] AND c_e)} over n codes
 // (indices c, coefficients coef), 64 codes per sweep. koff[i] holds the
-// packed chunk offsets of inv(i) (kappa_offsets4).
-template <int NKC, SweepShape SHAPE = kSweepWide>
+// packed chunk offsets of inv(i) (kappa_offsets4). Without ADD the first sweep
+// writes out instead unless `add` is set (n >= 1 then).
+template <int NKC, bool ADD = true>
 __device__ __forceinline__ void synthesise(Sweep &s, const uint32_t *c, const float *coef, int n, int t, int d,
-                                           const uint32_t *koff, float scale, float *out) {
+                                           const uint32_t *koff, float scale, float *out, bool add = true) {
     const int lane = threadIdx.x & 31;
     const int qn = (d + 31) / 32;
     for (int g0 = 0; g0 < n; g0 += 64) {
@@ -376,7 +386,7 @@ __device__ __forceinline__ void synthesise(Sweep &s, const uint32_t *c, const fl
         __syncwarp();
         sweep_build_values(s);
         __syncwarp();
-        sweep_accumulate_runs<NKC, SHAPE>(s, out, koff, d, scale);
+        sweep_accumulate_runs<NKC, ADD>(s, out, koff, d, scale, add || g0 > 0);
         __syncwarp();
     }
 }
