@@ -4,14 +4,14 @@
 // l-1 and keeps its top K_l distinct children; the code is every level's kept
 // set, level by level, each in (|z| descending, index ascending) order.
 //
-// Child scoring (Eq. 6) runs on the tcgen05 tensor cores. A block of 8 warps
-// owns 8 tokens. At level l its tensor-core rows are (token, parent slot):
+// Child scoring (Eq. 6) runs on the tcgen05 tensor cores. A block owns 8
+// tokens, two warps each (w and w + 8). At level l its tensor-core rows are (token, parent slot):
 // 16 slots per token (one M = 128 tile) when K_{l-1} <= 16, else 32 (two
 // tiles); its Delta_l columns are the level's generators, so one tcgen05.mma
 // of M = 128, N = Delta_l, K = 16 scores 128 x Delta_l children at once. Tile
 // t's TMEM lane quarter q holds the rows of token q + 4 t (32 slots), or of
 // tokens q and q + 4 (16 slots each), so that warp w reads its token's rows
-// from its own quarter. K runs over d in chunks of 64 coordinates, double
+// from its own quarter (as does warp w + 8). K runs over d in chunks of 64 coordinates, double
 // buffered:
 //  - A (128 x 64 bf16) is built in shared memory by the block's threads,
 //    each writing its row x (.) phi~_parent: the token's x pairs XOR the
@@ -20,9 +20,9 @@
 //    32-coordinate block hold coordinates (i, i + 16), whose sign bits one
 //    shift moves to the bf16 sign positions;
 //  - B (Delta_l x 64 bf16, the generators' +-1 signs in the same order) is
-//    one bulk copy of the plan's precomputed tile, issued by a tenth warp's
+//    one bulk copy of the plan's precomputed tile, issued by a further warp's
 //    lane 0 (the producer) once the MMAs that last read its stage are done;
-//  - a ninth warp's lane 0 issues the MMAs of a chunk once the 8 token
+//  - another warp's lane 0 issues the MMAs of a chunk once the 16 token
 //    warps have arrived on the A stage's mbarrier and the generator tile has
 //    landed, and commits them to an mbarrier that frees the chunk's buffers;
 //    scores accumulate in TMEM. The token warps build the next A stages
@@ -32,7 +32,8 @@
 // DPB_DEV_TIMEOUT and stops the block, which then waits (again bounded) for
 // its bulk copies and MMAs still in flight and frees its TMEM.
 //
-// Selection of a level (one warp per token, lane = parent slot): each lane
+// Selection of a level (two warps per token, each half of a row's columns,
+// lane = parent slot; half 0 ranks the keys of both and sorts): each lane
 // keeps the 4 largest of its row's group maxima (the largest key |z| of each
 // 8 consecutive children; at level 0, of each 8 of the lane's coordinates
 // lane + 32 j with consecutive j), the warp sorts the union and
@@ -52,10 +53,11 @@ namespace dpb {
 
 namespace {
 
-constexpr int kTokens = 8;      // tokens per block, one per warp
-constexpr int kThreads = (kTokens + 2) * 32;  // and a ninth warp, whose lane 0 issues the MMAs,
-constexpr int kIssuer = kTokens * 32;         // and a tenth, whose lane 0 copies the generator tiles
-constexpr int kProducer = (kTokens + 1) * 32;
+constexpr int kTokens = 8;                // tokens per block
+constexpr int kTokWarps = 2 * kTokens;    // token warps: w and w + 8 share token w
+constexpr int kIssuer = kTokWarps * 32;   // a further warp, whose lane 0 issues the MMAs,
+constexpr int kProducer = kIssuer + 32;   // and another, whose lane 0 copies the generator tiles
+constexpr int kThreads = kProducer + 32;
 constexpr int kRows = 32;       // tensor-core rows per token (parent slots)
 constexpr int kChunk = 64;      // coordinates per K chunk
 constexpr int kATile = 128 * kChunk * 2;  // one M = 128 tile of a chunk
@@ -88,15 +90,15 @@ struct Args {
 constexpr int kSelBytes = 8 * kSelCap;  // a warp's gathered (z, index) pairs
 
 struct Layout {
-    int a, b, xw, vh, g, w5, par, mbar, total;
+    int a, b, xw, vh, g, w5, par, ctl, mbar, total;
 };
 
-// The gathered candidates of the 8 warps share the generator-tile stages: a
+// The gathered candidates of the token warps share the generator-tile stages: a
 // level's selection starts once its MMAs are done and before the next
 // level's tiles are copied.
 __host__ __device__ inline Layout layout(int d, int levels, int kvh, int dmax, int nbs) {
     const int nblk = d / 32;
-    const int bbytes = nbs * dmax * 128 > kTokens * kSelBytes ? nbs * dmax * 128 : kTokens * kSelBytes;
+    const int bbytes = nbs * dmax * 128 > kTokWarps * kSelBytes ? nbs * dmax * 128 : kTokWarps * kSelBytes;
     Layout l;
     l.a = 0;
     l.b = l.a + 2 * 2 * kATile;  // 2 stages x 2 tiles
@@ -105,7 +107,8 @@ __host__ __device__ inline Layout layout(int d, int levels, int kvh, int dmax, i
     l.g = l.vh + kvh * nblk * 32 * 4;
     l.w5 = l.g + levels * 256 * 4;
     l.par = l.w5 + 32 * 4;
-    l.mbar = l.par + kTokens * kRows * 4;
+    l.ctl = l.par + kTokens * kRows * 4;
+    l.mbar = l.ctl + kTokens * 16;
     l.total = l.mbar + (2 * kMaxStages + 6) * 8 + 16;
     return l;
 }
@@ -193,10 +196,18 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32
 
 // ---- selection ---------------------------------------------------------------------
 
-struct WarpBufs {
-    uint32_t *par;   // [32] parents of the next level
-    float *z;        // [kSelCap]
-    uint32_t *id;    // [kSelCap]
+// A token's buffers, shared by its two warps (half h gathers into list h; the
+// keys of half 1 pass through list 1).
+struct TokenBufs {
+    uint32_t *par;     // [32] parents of the next level
+    float *z0, *z1;    // [kSelCap] gathered candidates of each half,
+    uint32_t *id0, *id1;  // their indices
+    uint32_t *ctl;     // [4] words handed between the halves
+    int half, bar;     // this warp's half; the pair's named barrier
+    __device__ __forceinline__ void sync() const {
+        __syncwarp();
+        asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory");
+    }
 };
 
 // One compare-exchange stage (size, stride) of a warp bitonic sort,
@@ -232,23 +243,28 @@ __device__ __forceinline__ void sort_stage64(uint64_t (&v)[R], int size, int str
     }
 }
 
-// Sorts the n (<= 32 R) gathered candidates as 64-bit words, drops repeated
+// Sorts the n (<= 32 R) gathered candidates (n0 of them in list 0) as 64-bit words, drops repeated
 // indices (equal candidates score equally, so copies sit side by side) and
 // writes the first K to code columns [col, col + K) of row `tok` (and the
 // parents of the next level). Returns the number of distinct candidates.
 template <int R>
-__device__ __forceinline__ int sort_keep(int n, int K, const WarpBufs &w, const Args &a, int64_t tok, int col,
-                                         bool par_out, bool write) {
+__device__ __forceinline__ int sort_keep(int n0, int n, int K, const TokenBufs &w, const Args &a, int64_t tok, int col,
+                                         bool par_out) {
     const int lane = threadIdx.x & 31;
     uint64_t v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int e = R * lane + r;
-        v[r] = e < n ? mmaenc::cword(w.z[e], w.id[e]) : 0ull;
+        v[r] = e < n0  ? mmaenc::cword(w.z0[e], w.id0[e])
+               : e < n ? mmaenc::cword(w.z1[e - n0], w.id1[e - n0])
+                       : 0ull;
     }
-#pragma unroll 1
+    // unrolled, stage by stage: a rolled loop's branches and run-time strides
+    // cost more latency than the shuffles (paper 3L step, 16,384 tokens, both
+    // sorts: 1,133 us rolled, 1,062 unrolled)
+#pragma unroll
     for (int size = 2; size <= 32 * R; size <<= 1)
-#pragma unroll 1
+#pragma unroll
         for (int stride = size / 2; stride > 0; stride >>= 1) sort_stage64<R>(v, size, stride);
     bool keep[R];
     uint32_t prev = __shfl_up_sync(kFull, mmaenc::cword_idx(v[R - 1]), 1);
@@ -268,19 +284,17 @@ __device__ __forceinline__ int sort_keep(int n, int K, const WarpBufs &w, const 
     }
     const int distinct = __shfl_sync(kFull, base, 31);
     base -= kept;
-    if (write) {
-        if (par_out) w.par[lane] = 0u;
-        __syncwarp();
+    if (par_out) w.par[lane] = 0u;
+    __syncwarp();
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (keep[r] && base < K) {
-                const uint32_t id = mmaenc::cword_idx(v[r]);
-                a.idx[tok * a.code_len + col + base] = (int32_t)id;
-                a.val[tok * a.code_len + col + base] = mmaenc::cword_z(v[r]);
-                if (par_out && base < kRows) w.par[base] = id;
-            }
-            base += keep[r];
+    for (int r = 0; r < R; ++r) {
+        if (keep[r] && base < K) {
+            const uint32_t id = mmaenc::cword_idx(v[r]);
+            a.idx[tok * a.code_len + col + base] = (int32_t)id;
+            a.val[tok * a.code_len + col + base] = mmaenc::cword_z(v[r]);
+            if (par_out && base < kRows) w.par[base] = id;
         }
+        base += keep[r];
     }
     __syncwarp();
     return distinct;
@@ -330,22 +344,24 @@ __device__ __forceinline__ uint32_t key_of_rank(const uint32_t (&v)[R], const in
     return __reduce_max_sync(kFull, mine);
 }
 
-// The top K distinct candidates of one token, as explained in the header.
-// `scan(f)` calls f(v, live, gend, index) for every candidate of this lane (the
-// first nlive lanes hold candidates), in
+// The top K distinct candidates of one token, as explained in the header, by
+// its two warps. `scan(f)` calls f(v, live, gend, index) for every candidate of
+// this lane in this warp's half of the row (the first nlive lanes hold
+// candidates), in
 // the same order each time and in step across the warp: v is its score before
 // the factor `scale` (> 0; the score is z = v scale), gend marks the last
 // candidate of a group (a group is live or not as a whole), and index() gives
 // its feature index. Scaling is monotone, so a group's largest |z| is its
-// largest |v| scaled once. Writes code columns [col, col + K) of row `tok`
-// and, when `par_out`, the kept indices as the next level's parents. Returns
-// the number of distinct candidates kept (< K only with the status bit set).
+// largest |v| scaled once. Half 0 ranks the keys of both halves and hands the
+// threshold to half 1; each gathers its half into its own list, and half 0
+// sorts both. Writes code columns [col, col + K) of row `tok` and, when
+// `par_out`, the kept indices as the next level's parents (fewer than K only
+// with the status bit set).
 template <class Scan>
-__device__ __forceinline__ int select_level(Scan scan, int nlive, float scale, int K, const WarpBufs &w,
-                                            const Args &a, int64_t tok, int col, bool par_out) {
+__device__ __forceinline__ void select_level(Scan scan, int nlive, float scale, int K, const TokenBufs &w,
+                                             const Args &a, int64_t tok, int col, bool par_out) {
     const int lane = threadIdx.x & 31;
     uint32_t top[4];
-    int nd = 0;  // distinct keys in the union
     // Group maxima first; when they hold fewer than K distinct keys (rows of
     // few children, or copies), every candidate's key instead.
     // each lane's 4 largest keys: of its group maxima, or (EVERY) of all its
@@ -368,39 +384,59 @@ __device__ __forceinline__ int select_level(Scan scan, int nlive, float scale, i
             }
         });
     };
-    // the union of each lane's first R keys, sorted, and the distinct key of a
-    // given rank in it: R = 2 when the nlive lanes that hold candidates give
-    // at least 2 K keys that way, else R = 4
-    uint32_t u2[2], u4[4];
-    int dr2[2], dr4[4];
-    const bool narrow = nlive >= K;
+    uint4 *xchg = reinterpret_cast<uint4 *>(w.z1);  // half 1's keys
+    uint32_t tau;
 #pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
+    for (int pass = 0;; ++pass) {
         if (pass == 0)
             lane_keys(std::false_type{});
         else
             lane_keys(std::true_type{});
-        if (narrow) {
-            u2[0] = top[0];
-            u2[1] = top[1];
-            nd = union_distinct<2>(u2, dr2);
-        } else {
-#pragma unroll
-            for (int r = 0; r < 4; ++r) u4[r] = top[r];
-            nd = union_distinct<4>(u4, dr4);
+        if (w.half == 1) xchg[lane] = make_uint4(top[0], top[1], top[2], top[3]);
+        w.sync();
+        if (w.half == 0) {
+            // the 4 largest of the lane's two sorted lists, sorted
+            const uint4 o = xchg[lane];
+            uint32_t x0 = max(top[0], o.w), x1 = max(top[1], o.z), x2 = max(top[2], o.y), x3 = max(top[3], o.x);
+            const uint32_t y0 = max(x0, x2), y2 = min(x0, x2), y1 = max(x1, x3), y3 = min(x1, x3);
+            top[0] = max(y0, y1);
+            top[1] = min(y0, y1);
+            top[2] = max(y2, y3);
+            top[3] = min(y2, y3);
+            // the union of each lane's first R keys, sorted, and the distinct key of a
+            // given rank in it: R = 2 when the nlive lanes that hold candidates give
+            // at least 2 K keys that way, else R = 4.
+            // tau = the union's distinct key of rank K: every key of the union is some
+            // candidate's, so K distinct candidates reach it and the level's top K
+            // distinct all do (the union's last distinct key when it holds fewer)
+            int nd;
+            if (nlive >= K) {
+                uint32_t u[2] = {top[0], top[1]};
+                int dr[2];
+                nd = union_distinct<2>(u, dr);
+                tau = key_of_rank<2>(u, dr, min(K, nd));
+            } else {
+                uint32_t u[4] = {top[0], top[1], top[2], top[3]};
+                int dr[4];
+                nd = union_distinct<4>(u, dr);
+                tau = key_of_rank<4>(u, dr, min(K, nd));
+            }
+            if (lane == 0) {
+                w.ctl[0] = tau;
+                w.ctl[1] = nd >= K || pass == 1;
+            }
         }
-        if (nd >= K) break;
+        w.sync();
+        tau = w.ctl[0];
+        if (w.ctl[1]) break;
     }
-    // tau = the union's distinct key of rank K: every key of the union is some
-    // candidate's, so K distinct candidates reach it and the level's top K
-    // distinct all do (the union's last distinct key when it holds fewer)
-    const int target = min(K, nd);
-    uint32_t tau = narrow ? key_of_rank<2>(u2, dr2, target) : key_of_rank<4>(u4, dr4, target);
     if (tau == 0u) tau = 1u;
     // key(z) + 1 >= tau exactly when |z| >= the float with bits tau - 1
     const float tf = __uint_as_float(tau - 1u);
     // gather every candidate at or above tau, warp-interleaved in scan order
     // (one pass: positions come from the running ballot counts)
+    float *lz = w.half ? w.z1 : w.z0;
+    uint32_t *lid = w.half ? w.id1 : w.id0;
     int n = 0;
     scan([&](float v, bool live, bool, auto index) {
         const float z = v * scale;
@@ -409,22 +445,26 @@ __device__ __forceinline__ int select_level(Scan scan, int nlive, float scale, i
         if (mb) {  // rare: most candidates fall short of tau
             const int pos = n + __popc(mb & ((1u << lane) - 1u));
             if (take && pos < kSelCap) {
-                w.z[pos] = z;
-                w.id[pos] = index();
+                lz[pos] = z;
+                lid[pos] = index();
             }
             n += __popc(mb);
         }
     });
+    if (w.half == 1 && lane == 0) w.ctl[2] = (uint32_t)n;
+    w.sync();
+    if (w.half == 1) return;
+    const int n0 = min(n, kSelCap);
+    n += (int)w.ctl[2];
     if (n > kSelCap) {
         set_status(a.status, DPB_DEV_SHORT_CODE);
         n = kSelCap;
     }
-    __syncwarp();
     // the narrowest sort that holds them: 32, 64, 128 or 256 words
-    const int distinct = n <= 32    ? sort_keep<1>(n, K, w, a, tok, col, par_out, true)
-                         : n <= 64  ? sort_keep<2>(n, K, w, a, tok, col, par_out, true)
-                         : n <= 128 ? sort_keep<4>(n, K, w, a, tok, col, par_out, true)
-                                    : sort_keep<8>(n, K, w, a, tok, col, par_out, true);
+    const int distinct = n <= 32    ? sort_keep<1>(n0, n, K, w, a, tok, col, par_out)
+                         : n <= 64  ? sort_keep<2>(n0, n, K, w, a, tok, col, par_out)
+                         : n <= 128 ? sort_keep<4>(n0, n, K, w, a, tok, col, par_out)
+                                    : sort_keep<8>(n0, n, K, w, a, tok, col, par_out);
     if (distinct < K) {
         set_status(a.status, DPB_DEV_SHORT_CODE);
         for (int e = distinct + lane; e < K; e += 32) {
@@ -433,7 +473,6 @@ __device__ __forceinline__ int select_level(Scan scan, int nlive, float scale, i
         }
     }
     __syncwarp();
-    return distinct;
 }
 
 __device__ __forceinline__ float standardise(float s, uint32_t c, const Args &a, int32_t *status) {
@@ -485,10 +524,16 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
     // full_b[stages], mma_done[stages], a_full[2 + 4]
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + lay.mbar);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mbar + 2 * kMaxStages + 6);
-    WarpBufs wb;
-    wb.par = reinterpret_cast<uint32_t *>(smem + lay.par) + warp * kRows;
-    wb.z = reinterpret_cast<float *>(sB + warp * kSelBytes);
-    wb.id = reinterpret_cast<uint32_t *>(sB + warp * kSelBytes + 4 * kSelCap);
+    const int tw = warp & (kTokens - 1);  // the token of this (token) warp
+    TokenBufs wb;
+    wb.par = reinterpret_cast<uint32_t *>(smem + lay.par) + tw * kRows;
+    wb.z0 = reinterpret_cast<float *>(sB + tw * kSelBytes);
+    wb.z1 = reinterpret_cast<float *>(sB + (tw + kTokens) * kSelBytes);
+    wb.id0 = reinterpret_cast<uint32_t *>(wb.z0 + kSelCap);
+    wb.id1 = reinterpret_cast<uint32_t *>(wb.z1 + kSelCap);
+    wb.ctl = reinterpret_cast<uint32_t *>(smem + lay.ctl) + 4 * tw;
+    wb.half = warp >> 3;
+    wb.bar = 1 + tw;
     for (int i = tid; i < a.kvh * nblk * 32; i += blockDim.x) vh[i] = a.VH2[i];
     for (int i = tid; i < L * 256; i += blockDim.x) gs[i] = a.G[(i >> 8) * DPB_MAX_CHILDREN + (i & 255)];
     if (tid < 32) {
@@ -501,7 +546,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar + i)));
         for (int i = 0; i < 6; ++i)  // an A stage is built once each of the token warps arrives
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar + 2 * kMaxStages + i)),
-                         "r"(kTokens));
+                         "r"(kTokWarps));
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (warp == 0) {
@@ -542,17 +587,17 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
     };
     const uint32_t lo_mask = (1u << a.t) - 1u;
     const int64_t ngroups = (a.T + kTokens - 1) / kTokens;
-    uint16_t *xh = reinterpret_cast<uint16_t *>(xw + warp * nblk * 16);
+    uint16_t *xh = reinterpret_cast<uint16_t *>(xw + tw * nblk * 16);
 
     for (int64_t grp = blockIdx.x; grp < ngroups && !failed; grp += gridDim.x) {
-        const int64_t tok = grp * kTokens + warp;
-        const bool live = warp < kTokens && tok < a.T;
+        const int64_t tok = grp * kTokens + tw;
+        const bool live = warp < kTokWarps && tok < a.T;
         // ---- the row in the pair layout: word m*16 + i = (x[32m+i], x[32m+i+16]); |x|; level 0 ----
         if (live) {
             const uint4 *row = reinterpret_cast<const uint4 *>(a.x + tok * d);
             float ss = 0.f;
-#pragma unroll 4  // the row's loads in flight together (4 chunks per lane at d = 1024)
-            for (int ch = lane; ch < d / 8; ch += 32) {
+#pragma unroll 2  // the row's loads in flight together (2 chunks per lane at d = 1024)
+            for (int ch = lane + 32 * wb.half; ch < d / 8; ch += 64) {
                 const uint4 v = row[ch];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
@@ -564,12 +609,15 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
                 }
             }
             ss = warp_sum(ss);
-            if (lane == 0 && a.xnorm) a.xnorm[tok] = sqrtf(ss);
-            __syncwarp();
-            // a lane's coordinates lane + 32 j in groups of 8 consecutive j (d is
+            if (lane == 0 && wb.half == 1) wb.ctl[3] = __float_as_uint(ss);
+            wb.sync();  // the row is staged by both halves
+            if (lane == 0 && wb.half == 0 && a.xnorm) a.xnorm[tok] = sqrtf(ss + __uint_as_float(wb.ctl[3]));
+            // this half's blocks of 32 coordinates, in whole groups; a lane's coordinates lane + 32 j in groups of 8 consecutive j (d is
             // a multiple of 64, so every lane has the same count)
+            const int hb0 = ((nblk + 7) / 8 + 1) / 2 * 8;
+            const int i0 = wb.half ? 32 * hb0 : 0, i1 = wb.half ? d : min(d, 32 * hb0);
             auto scan0 = [&](auto f) {
-                for (int i = lane; i < d; i += 32) {
+                for (int i = i0 + lane; i < i1; i += 32) {
                     const int m = i >> 5, wl = i & 31;
                     const float xv = __uint_as_float((uint32_t)xh[(m * 16 + (wl & 15)) * 2 + (wl >> 4)] << 16);
                     f(standardise(xv, (uint32_t)i, a, nullptr), true, (m & 7) == 7 || i + 32 >= d,
@@ -577,9 +625,9 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
                 }
             };
             if (a.mu)
-                for (int i = lane; i < d; i += 32) standardise(0.f, (uint32_t)i, a, a.status);
+                for (int i = i0 + lane; i < i1; i += 32) standardise(0.f, (uint32_t)i, a, a.status);
             select_level(scan0, 32, 1.f, a.kl[0], wb, a, tok, a.off[0], L > 1);  // d >= 64: every lane holds 2+
-        } else if (warp < kTokens) {
+        } else if (warp < kTokWarps) {
             wb.par[lane] = 0u;
             __syncwarp();
         }
@@ -588,8 +636,8 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
         for (int l = 1; l < L && !failed; ++l) {
             const int P = a.kl[l - 1], D = a.delta[l], nch = d / kChunk;
             const int pp = P <= 16 ? 16 : 32, ntiles = pp / 16;  // slots per token, M = 128 tiles
-            // this thread builds block half hb of row rr of each tile
-            const int rr = tid & 127, hb = tid >> 7;
+            // this thread builds half qh of block hb of the chunk, in row rr of each tile
+            const int rr = tid & 127, hb = tid >> 8, qh = (tid >> 7) & 1;
             // A row that is no live parent (a slot past K_{l-1}, a token past T)
             // takes parent 0 and whatever x its buffer holds: the selection
             // reads only live rows, and an MMA row depends on its own A row only
@@ -696,7 +744,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
                             const uint4 *xs = reinterpret_cast<const uint4 *>(ixt[tt] + m * 16);
                             uint8_t *At = As + tt * kATile;
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) {
+                            for (int q = 2 * qh; q < 2 * qh + 2; ++q) {
                                 const uint4 xv = xs[q];
                                 const int sh = 15 - 4 * q;
                                 uint4 av;
@@ -736,12 +784,13 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
             // TMEM, so the selection's three passes gather no tables. Warp w
             // takes quarter w % 4 (all 32 rows; with 16 slots a quarter holds
             // tokens q and q + 4) of tile w / 4, or with one tile half w / 4 of
-            // the columns: all eight warps keep table loads in flight.
+            // the columns: all sixteen warps keep table loads in flight.
             if (a.mu) {
-                if (warp < kTokens) {
-                    const int q = warp & 3, tile = ntiles == 2 ? warp >> 2 : 0;
-                    const int half = ((D + 31) / 32 + 1) / 2 * 32;  // whole 32-column loads
-                    const int cb = ntiles == 2 ? 0 : (warp >> 2) * half, ce = ntiles == 2 ? D : min(D, cb + half);
+                if (warp < kTokWarps) {
+                    const int q = warp & 3, tile = ntiles == 2 ? (warp >> 2) & 1 : 0;
+                    const int parts = ntiles == 2 ? 2 : 4, part = ntiles == 2 ? warp >> 3 : warp >> 2;
+                    const int cols = ((D + 31) / 32 + parts - 1) / parts * 32;  // whole 32-column loads
+                    const int cb = part * cols, ce = min(D, cb + cols);
                     const int tokw = pp == 32 ? q + 4 * tile : q + 4 * (lane >> 4);
                     const int slot = pp == 32 ? lane : lane & 15;
                     const bool ok = grp * kTokens + tokw < a.T && slot < P;
@@ -753,18 +802,20 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
                 __syncthreads();
                 asm volatile("tcgen05.fence::after_thread_sync;");
             }
-            // ---- the level's selection, one warp per token ----
+            // ---- the level's selection, two warps per token ----
             if (live) {
-                // this warp's rows: tile (warp / 4 when 32 slots), quarter warp % 4,
-                // lanes [base, base + pp) of it
-                const int tile = pp == 32 ? warp >> 2 : 0, base = pp == 16 ? 16 * (warp >> 2) : 0;
+                // this token's rows: tile (tw / 4 when 32 slots), quarter tw % 4,
+                // lanes [base, base + pp) of it; this warp's half of the columns
+                const int tile = pp == 32 ? tw >> 2 : 0, base = pp == 16 ? 16 * (tw >> 2) : 0;
+                const int half = ((D + 31) / 32 + 1) / 2 * 32;
+                const int cb = wb.half * half, ce = wb.half ? D : min(D, half);
                 const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 256u * tile;
                 const int slot = lane - base;
                 const bool rv = slot >= 0 && slot < pp && slot < P;
                 const uint32_t p = rv ? wb.par[slot] : 0u;
                 const float scale = a.mu ? 1.f : a.inv_sqrt_d;  // TMEM holds z, or s sqrt(d)
                 auto scanl = [&](auto f) {
-                    for (int c0 = 0; c0 < D; c0 += 32) {
+                    for (int c0 = cb; c0 < ce; c0 += 32) {
                         uint32_t v[32];
                         tmem_ld32(taddr + c0, v);
                         // D is a multiple of 16: columns c0 + 16 .. c0 + 31 exist as a
