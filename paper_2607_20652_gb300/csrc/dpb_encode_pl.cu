@@ -475,10 +475,6 @@ __device__ __forceinline__ void select_level(Scan scan, int nlive, float scale, 
     __syncwarp();
 }
 
-__device__ __forceinline__ float standardise(float s, uint32_t c, const Args &a, int32_t *status) {
-    return a.mu ? zscore(s, c, a.mu, a.sigma, a.tab, status) : s;
-}
-
 // Standardised scores of one warp's TMEM rows, columns [cb, ce) (Delta = D
 // children of parent p, live when ok): z = (s / sqrt(d) - mu_c) / sigma_c in
 // place of s. Four columns' table loads are in flight at a time. Not inlined:
@@ -504,6 +500,35 @@ __device__ __noinline__ void standardise_cols(const float *mu, const float *sigm
             }
         }
         tmem_st32(taddr + c0, v);
+    }
+    if (bad) set_status(status, DPB_DEV_BAD_SIGMA);
+}
+
+// Coordinate i of a row in the pair layout.
+__device__ __forceinline__ float x_of(const uint16_t *xh, int i) {
+    const int m = i >> 5, wl = i & 31;
+    return __uint_as_float((uint32_t)xh[(m * 16 + (wl & 15)) * 2 + (wl >> 4)] << 16);
+}
+
+// Level 0 with tables: zb[i] = (x_i - mu_i) / sigma_i of this lane's
+// coordinates i0 + lane + 32 j < i1, eight table loads in flight. The
+// selection's two scans, which waited for every load in turn, and a third pass
+// for the sigma check took 39 thousand cycles of a group's 158 at d = 2048; this
+// and the scans take 20. Not inlined, like standardise_cols.
+__device__ __noinline__ void standardise_row(const float *mu, const float *sigma, const float2 *tab, int32_t *status,
+                                             const uint16_t *xh, float *zb, int i0, int i1) {
+    bool bad = false;
+    for (int ib = i0 + (int)(threadIdx.x & 31); ib < i1; ib += 256) {
+        float2 e[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            e[j] = ib + 32 * j < i1 ? ztab((uint32_t)(ib + 32 * j), mu, sigma, tab) : make_float2(0.f, 1.f);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (ib + 32 * j < i1) {
+                zb[ib + 32 * j] = (x_of(xh, ib + 32 * j) - e[j].x) * e[j].y;
+                bad |= zbad(e[j].y);
+            }
     }
     if (bad) set_status(status, DPB_DEV_BAD_SIGMA);
 }
@@ -616,16 +641,17 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
             // a multiple of 64, so every lane has the same count)
             const int hb0 = ((nblk + 7) / 8 + 1) / 2 * 8;
             const int i0 = wb.half ? 32 * hb0 : 0, i1 = wb.half ? d : min(d, 32 * hb0);
-            auto scan0 = [&](auto f) {
-                for (int i = i0 + lane; i < i1; i += 32) {
-                    const int m = i >> 5, wl = i & 31;
-                    const float xv = __uint_as_float((uint32_t)xh[(m * 16 + (wl & 15)) * 2 + (wl >> 4)] << 16);
-                    f(standardise(xv, (uint32_t)i, a, nullptr), true, (m & 7) == 7 || i + 32 >= d,
-                      [&] { return (uint32_t)i; });
-                }
-            };
+            // z once per coordinate, as fp32, into the A stages (idle at level 0; 8
+            // tokens x 2048 words at most)
+            float *zb = reinterpret_cast<float *>(sA) + tw * d;
             if (a.mu)
-                for (int i = i0 + lane; i < i1; i += 32) standardise(0.f, (uint32_t)i, a, a.status);
+                standardise_row(a.mu, a.sigma, a.tab, a.status, xh, zb, i0, i1);
+            else
+                for (int i = i0 + lane; i < i1; i += 32) zb[i] = x_of(xh, i);
+            auto scan0 = [&](auto f) {  // (a lane reads back its own z only)
+                for (int i = i0 + lane; i < i1; i += 32)
+                    f(zb[i], true, ((i >> 5) & 7) == 7 || i + 32 >= d, [&] { return (uint32_t)i; });
+            };
             select_level(scan0, 32, 1.f, a.kl[0], wb, a, tok, a.off[0], L > 1);  // d >= 64: every lane holds 2+
         } else if (warp < kTokWarps) {
             wb.par[lane] = 0u;
@@ -783,8 +809,9 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
             // ---- standardised scores, once per candidate (§2.2): z replaces s in
             // TMEM, so the selection's three passes gather no tables. Warp w
             // takes quarter w % 4 (all 32 rows; with 16 slots a quarter holds
-            // tokens q and q + 4) of tile w / 4, or with one tile half w / 4 of
-            // the columns: all sixteen warps keep table loads in flight.
+            // tokens q and q + 4) of tile (w / 4) % 2 and half w / 8 of the
+            // columns, or with one tile their quarter w / 4: all sixteen warps
+            // keep table loads in flight.
             if (a.mu) {
                 if (warp < kTokWarps) {
                     const int q = warp & 3, tile = ntiles == 2 ? (warp >> 2) & 1 : 0;
