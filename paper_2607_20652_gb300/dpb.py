@@ -121,13 +121,19 @@ def _check(status: int):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+# The current stream's handle without building a torch.cuda.Stream (3 us a
+# call on a Grace core, four calls to a forward and backward).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+    (lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return _raw_stream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 _DTYPES = {"f32": (F32, torch.float32), "fp32": (F32, torch.float32), "float32": (F32, torch.float32),
@@ -184,6 +190,8 @@ class Plan:
         self.n_features = 1 << self.config["bits"][self.config["levels"] - 1]  # 2^N
         self.d = d
         self.torch_dtype = _DTYPES[dtype][1]
+        self._ws_bytes = self.workspace_size(0)  # the same for every T
+        self._ws_cache = {}
 
     def __del__(self):
         h = getattr(self, "_h", None)
@@ -222,15 +230,14 @@ class Plan:
         kept with the plan (calls on one stream run in order, so they may
         share it; its status bits accumulate until read and cleared)."""
         dev = torch.device(device)
-        s = stream if stream is not None else torch.cuda.current_stream(dev)
-        key = (dev.index if dev.index is not None else torch.cuda.current_device(), s.cuda_stream)
-        cache = self.__dict__.setdefault("_ws_cache", {})
-        ws = cache.get(key)
-        if ws is None or ws.numel() < self.workspace_size(T):
+        index = dev.index if dev.index is not None else torch.cuda.current_device()
+        key = (index, stream.cuda_stream if stream is not None else _raw_stream(index))
+        ws = self._ws_cache.get(key)
+        if ws is None or ws.numel() < self._ws_bytes:
             # allocated and zeroed on the stream the calls use, so the first
             # kernel cannot start before the fill ends
-            with torch.cuda.stream(s):
-                ws = cache[key] = self.workspace(T, dev)
+            with torch.cuda.stream(stream if stream is not None else torch.cuda.current_stream(dev)):
+                ws = self._ws_cache[key] = self.workspace(T, dev)
         return ws
 
     def status(self, device=None, stream=None, clear: bool = True) -> int:
@@ -239,7 +246,7 @@ class Plan:
         dev = torch.device(device or "cuda")
         s = stream if stream is not None else torch.cuda.current_stream(dev)
         key = (dev.index if dev.index is not None else torch.cuda.current_device(), s.cuda_stream)
-        ws = self.__dict__.get("_ws_cache", {}).get(key)
+        ws = self._ws_cache.get(key)
         return 0 if ws is None else workspace_status(ws, clear=clear, stream=s)
 
 

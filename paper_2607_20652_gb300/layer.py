@@ -21,42 +21,54 @@ from . import dpb
 
 
 class _DPBFunction(torch.autograd.Function):
+    # x of any leading shape: the rows are taken here, outside the graph, so
+    # that no reshape node runs in the backward
     @staticmethod
     def forward(ctx, x, layer):
-        T = x.shape[0]
+        rows = x.reshape(-1, layer.d).contiguous()
+        T = rows.shape[0]
         ws = layer._workspace(T, x.device)
-        stream = torch.cuda.current_stream(x.device)
+        stream = layer._stream(x.device)
         ev = layer._events("forward")
         r = torch.empty((T, layer.d), dtype=torch.float32, device=x.device)  # kept for the backward
-        idx, val, xn, y = dpb.forward(layer.plan, x, layer.mu, layer.sigma, workspace=ws, stream=stream, r_out=r)
+        idx, val, xn, y = dpb.forward(layer.plan, rows, layer.mu, layer.sigma, workspace=ws, stream=stream, r_out=r)
         if layer.ema is not None and layer.training:
-            rows = dpb.sample_rows(T, layer.ema_rows, layer._gen, x.device)
-            dpb.stats_accumulate(layer.plan, x, rows, layer._acc, mu=layer.mu, sigma=layer.sigma, workspace=ws,
+            sample = dpb.sample_rows(T, layer.ema_rows, layer._gen, x.device)
+            dpb.stats_accumulate(layer.plan, rows, sample, layer._acc, mu=layer.mu, sigma=layer.sigma, workspace=ws,
                                  stream=stream)
         if ev:
-            ev[1].record(stream)
-        ctx.save_for_backward(x, idx, val, r)
+            ev[1].record()
+        ctx.save_for_backward(rows, idx, val, r)
         ctx.layer = layer
-        layer.last_code = (idx, val)
-        return y
+        layer.__dict__["last_code"] = (idx, val)  # (a plain attribute: Module.__setattr__ looks for parameters)
+        return y.view(x.shape)
 
     @staticmethod
     def backward(ctx, gy):
-        x, idx, val, r = ctx.saved_tensors
+        rows, idx, val, r = ctx.saved_tensors
         layer = ctx.layer
-        gy = gy.contiguous().to(x.dtype)
-        ws = layer._workspace(x.shape[0], x.device)
-        stream = torch.cuda.current_stream(x.device)
+        shape = gy.shape
+        gy = gy.reshape(rows.shape).contiguous().to(rows.dtype)
+        ws = layer._workspace(rows.shape[0], rows.device)
+        stream = layer._stream(rows.device)
         ev = layer._events("backward")
-        gx, gv = dpb.backward(layer.plan, x, idx, val, gy, layer.sigma, workspace=ws, stream=stream, r=r)
+        gx, gv = dpb.backward(layer.plan, rows, idx, val, gy, layer.sigma, workspace=ws, stream=stream, r=r)
         if layer.ema is not None and layer.training:
             dpb.ema_step(lambda a: None,
                          lambda a: dpb.stats_update(layer.plan, a, layer.ema, layer.mu, layer.sigma, stream=stream),
                          layer._acc, layer.group)
         if ev:
-            ev[1].record(stream)
-        layer.last_grad_val = gv
-        return gx, None
+            ev[1].record()
+        layer.__dict__["last_grad_val"] = gv
+        return gx.view(shape), None
+
+
+class _RawStream:
+    """A stream handle with the one attribute the calls read."""
+    __slots__ = ("cuda_stream",)
+
+    def __init__(self, handle):
+        self.cuda_stream = handle
 
 
 class DPBLayer(torch.nn.Module):
@@ -92,10 +104,15 @@ class DPBLayer(torch.nn.Module):
         self.last_grad_val = None
 
     def _workspace(self, T, device):
-        n = self.plan.workspace_size(T)
+        n = self.plan._ws_bytes
         if self._ws is None or self._ws.numel() < n or self._ws.device != device:
             self._ws = torch.zeros(n, dtype=torch.uint8, device=device)
         return self._ws
+
+    def _stream(self, device):
+        if device.type != "cuda":
+            raise ValueError(f"x must be on a CUDA device, not {device}")
+        return _RawStream(dpb._raw_stream(device.index))
 
     def _events(self, which):
         if self.timing is None:
@@ -106,8 +123,6 @@ class DPBLayer(torch.nn.Module):
         return ev
 
     def forward(self, x):
-        shape = x.shape
-        if shape[-1] != self.d:
-            raise ValueError(f"last dimension {shape[-1]} != d = {self.d}")
-        rows = x.reshape(-1, self.d).to(self.plan.torch_dtype).contiguous()
-        return _DPBFunction.apply(rows, self).view(shape)
+        if x.shape[-1] != self.d:
+            raise ValueError(f"last dimension {x.shape[-1]} != d = {self.d}")
+        return _DPBFunction.apply(x.to(self.plan.torch_dtype), self)
