@@ -355,7 +355,7 @@ __device__ __forceinline__ void warp_sort_desc_runs(W (&v)[R]) {
 // before it) and how many entrants are ahead of each entrant (those in
 // earlier gaps, and those of its own gap that are larger, compared directly).
 template <int KPL>
-__device__ __noinline__ void merge_sorted(uint64_t *L, int k, uint64_t *E, int m, uint32_t *beam) {
+__device__ __forceinline__ void merge_sorted_body(uint64_t *L, int k, uint64_t *E, int m, uint32_t *beam) {
     const int lane = threadIdx.x & 31;
     const int top = 1 << (31 - __clz(k));  // the largest power of 2 <= k
     if (m >= 8 && m <= 32) {
@@ -454,10 +454,16 @@ __device__ __noinline__ void merge_sorted(uint64_t *L, int k, uint64_t *E, int m
     }
 }
 
+// One copy of the merge for all its callers in a kernel.
+template <int KPL>
+__device__ __noinline__ void merge_sorted(uint64_t *L, int k, uint64_t *E, int m, uint32_t *beam) {
+    merge_sorted_body<KPL>(L, k, E, m, beam);
+}
+
 // Gathers the candidate words c[] (4 per lane, 0 = none) that are ahead of the
 // list's k-th word into E (capacity >= 128) and merges them into L. Returns
-// the number of entrants.
-template <int KPL>
+// the number of entrants. INLINE: the merge's code in place.
+template <int KPL, bool INLINE = false>
 __device__ __forceinline__ int merge_entrants(uint64_t *L, int k, uint64_t *E, const uint64_t (&c)[4],
                                               uint32_t *beam) {
     const uint64_t tau = L[k - 1];
@@ -470,7 +476,10 @@ __device__ __forceinline__ int merge_entrants(uint64_t *L, int k, uint64_t *E, c
         m += __popc(mb);
     }
     __syncwarp();
-    merge_sorted<KPL>(L, k, E, m, beam);
+    if constexpr (INLINE)
+        merge_sorted_body<KPL>(L, k, E, m, beam);
+    else
+        merge_sorted<KPL>(L, k, E, m, beam);
     return m;
 }
 
@@ -929,7 +938,10 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
                 const uint4 *xb = reinterpret_cast<const uint4 *>(xt + (WIDE ? 0 : nblk * 16)) + q4;
                 const uint4 *fr = reinterpret_cast<const uint4 *>(frag) + lane;
                 const int sh = 15 - q4;
-#pragma unroll 2
+                // (4 blocks a trip pay with a warp per token: sweep step at beam 16
+                // 1,144 us against 1,133; with two tokens 670 against 681)
+                constexpr int kTrip = WIDE ? 4 : 2;
+#pragma unroll kTrip
                 for (int m = 0; m < nblk; ++m) {
                     const uint4 va = xa[m * 4], vb = xb[m * 4];
                     const uint2 sg = sgn[m * 8 + slot];
@@ -1063,7 +1075,11 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
                 }
                 pcur = p1;
                 const bool next = l + 1 < L;
-                const int m = merge_entrants<KPL>(Lt, k, E, c, next && !WIDE ? bt : nullptr);
+                // the merge in place, except for lists of 33 to 64 words, whose
+                // loop the call keeps small: 65,536 tokens forward at k = 64 took 670
+                // us with the call and 679 without, at k = 128 1,060 and 1,031, and
+                // the sweep step at beam 16, k = 128 1,144 and 1,093
+                const int m = merge_entrants<KPL, WIDE || KPL != 2>(Lt, k, E, c, next && !WIDE ? bt : nullptr);
                 if constexpr (WIDE) {
                     if (tk == 0) {
 #pragma unroll
