@@ -398,12 +398,34 @@ __global__ void __launch_bounds__(kSearchThreads, 1) stats_search_kernel(StatsAr
 
 // ---- the EMA step -----------------------------------------------------------------
 
+// 1 / n and sqrt(v) in fp64 by Newton's iteration from an fp32 estimate (an
+// error of 2^-22 squares to 2^-44 and then below fp64's): this chip has about
+// two fp64 lanes per SM and clock, and the library's division and root take some
+// 120 fp64 instructions a feature where these take 20. Both are within a few
+// fp64 units of the exact value, before a rounding to fp32.
+__device__ __forceinline__ double newton_rcp(double n) {
+    double r = (double)(1.0f / (float)n);
+    r = fma(r, fma(-n, r, 1.0), r);
+    return fma(r, fma(-n, r, 1.0), r);
+}
+__device__ __forceinline__ double newton_sqrt(double v) {
+    if (!(v > 1e-30 && v < 1e30)) return sqrt(v);  // outside fp32's comfortable range
+    double r = (double)rsqrtf((float)v);           // r -> 1 / sqrt(v): r += r (1 - v r^2) / 2
+    r = fma(0.5 * r, fma(-v * r, r, 1.0), r);
+    r = fma(0.5 * r, fma(-v * r, r, 1.0), r);
+    const double y = v * r;
+    return fma(0.5 * r, fma(-y, y, v), y);
+}
+
 // A block reads the counts of kUpdFeatures features and lists the touched ones,
-// so that their fp64 arithmetic (slow on this chip, two divisions and a root
-// each) runs in full warps: with a feature per thread nearly every warp held
-// one touched feature of a sparse batch and ran it all (2^20 features, 3%
-// touched: 16.8 us, 6.6 now).
-constexpr int kUpdFeatures = 1024;
+// so that their fp64 arithmetic runs in full warps (a feature per thread would
+// run it in nearly every warp of a sparse batch). Small blocks: level 0 touches
+// every basis coordinate, and a block of 1,024 features left all their
+// arithmetic to one SM. 2^20 features, 3% touched: 16.8 us with a feature per
+// thread and library arithmetic; the standardised step of 8,192 tokens 298 us
+// with blocks of 1,024 and library arithmetic, 284 with blocks of 512 and 282
+// with 256 of these.
+constexpr int kUpdFeatures = 256;
 __global__ void __launch_bounds__(256) stats_update_kernel(double *acc, int64_t m, double alpha, float *mu,
                                                            float *sigma) {
     __shared__ uint16_t list[kUpdFeatures];
@@ -424,12 +446,13 @@ __global__ void __launch_bounds__(256) stats_update_kernel(double *acc, int64_t 
         for (int e = threadIdx.x; e < count; e += 256) {
             const int64_t i = base + list[e];
             const double n = acc[i], s = acc[m + i], q = acc[2 * m + i];
-            const double mean = s / n;
+            const double rn = newton_rcp(n);
+            const double mean = s * rn;
             const double mu0 = mu[i];
             mu[i] = (float)(mu0 + alpha * (mean - mu0));
             if (n >= 1.5) {
-                const double var = q / n - mean * mean;
-                const double v = sqrt(var > 0.0 ? var : 0.0);
+                const double var = q * rn - mean * mean;
+                const double v = var > 0.0 ? newton_sqrt(var) : 0.0;
                 const double sg0 = sigma[i];
                 sigma[i] = (float)(sg0 + alpha * (v - sg0));
             }
