@@ -283,3 +283,63 @@ def test_bad_sigma_is_flagged_not_faulted():
     ws = pl.workspace(16, dev)
     dpb.encode(pl, x2, torch.zeros(pl.n_features, device=dev), sg2, workspace=ws)
     assert dpb.workspace_status(ws) & dpb.DEV_BAD_SIGMA
+
+
+def _update_zeroed(n, s, q):
+    """One EMA step of zero tables at alpha = 1/2 on the given sums: (2 mu, 2 sigma)
+    as fp64, i.e. the means and deviations to fp32 rounding, and exact zeros."""
+    plan, _ = _pair(dtype="f32", d=64, levels=3, m_bits=12, children=16, beam=4, k=8)
+    acc = np.zeros((3, 1 << 12))
+    acc[:, :len(n)] = n, s, q
+    dev = torch.device("cuda")
+    mu, sg = torch.zeros(1 << 12, device=dev), torch.zeros(1 << 12, device=dev)
+    dpb.stats_update(plan, torch.from_numpy(acc).to(dev), 0.5, mu, sg)
+    return [2.0 * t.cpu().numpy().astype(np.float64)[:len(n)] for t in (mu, sg)]
+
+
+def test_ema_update_of_equal_scores_is_exact():
+    # n equal scores c of 8 significant bits: s = n c and q = n c^2 are exact, so
+    # mean = c and deviation = 0 exactly whatever n
+    g = inputs.rng(26)
+    n = np.resize([2.0, 3, 5, 7, 21, 25, 31, 49, 1000, 8192, 65537], 4000)
+    c = inputs.to_bf16(g.uniform(0.5, 8.0, 4000).astype(np.float32)).astype(np.float64)
+    mean, dev = _update_zeroed(n, n * c, n * c * c)
+    assert np.array_equal(mean, c) and not dev.any()
+    # the same through the column pass and the sampled search: 25 equal rows (a
+    # 24-bit score's square summed 25 times stays within 53 bits)
+    plan, _ = _pair(d=64, levels=3, m_bits=12, children=16, beam=4, k=8)
+    x = torch.from_numpy(inputs.gaussian_rows(1, 64, 27)).cuda().to(torch.bfloat16).expand(25, 64).contiguous()
+    acc = dpb.stats_buffer(plan)
+    dpb.stats_accumulate(plan, x, torch.arange(25, dtype=torch.int32, device="cuda"), acc)
+    touched = acc[0] > 0
+    assert int(touched.sum()) > 64 + 100 and bool((acc[0][touched] == 25).all())
+    mu, sg = torch.zeros(1 << 12, device="cuda"), torch.zeros(1 << 12, device="cuda")
+    dpb.stats_update(plan, acc, 0.5, mu, sg)
+    assert torch.equal(2 * mu[:64], x[0].float()) and not sg.any().item()
+
+
+def test_ema_update_deviations_against_exact_arithmetic():
+    # Means of 10^3 to 10^7 deviations: q / n and s / n rounded once each leave
+    # the difference q / n - mean^2 within 2^-53 (q / n + 2 mean^2) of the exact
+    # one (second-order terms and its own rounding: 2^-50 of the bound, 2^-52 of
+    # itself), and the fp32 result within 2^-24 of its root (2^-23 of it).
+    from fractions import Fraction
+    g = inputs.rng(28)
+    n = g.integers(2, 100000, 2000).astype(np.float64)
+    mean = 10.0 ** g.uniform(3, 7, 2000)
+    s = n * mean
+    q = n * (mean * mean + g.uniform(0.5, 2.0, 2000))
+    got = _update_zeroed(n, s, q)[1]
+    for ni, si, qi, v in zip(n, s, q, got):
+        a, m = Fraction(qi) / Fraction(ni), Fraction(si) / Fraction(ni)
+        exact, bound = a - m * m, float(a + 2 * m * m) * 2.0 ** -53 * (1 + 2.0 ** -50)
+        if float(exact) > 4 * bound:
+            assert abs(float(Fraction(v) ** 2 - exact)) <= bound + float(exact + Fraction(bound)) * (2.0 ** -23 + 2.0 ** -46)
+    # roots of variances across fp64's range, both sides of the fast root's own
+    var = np.array([1e-80, 0.99e-30, 1.01e-30, 3e-30, 1e-9, 0.3, 2.0, 1e9, 0.99e30, 1.01e30, 1e60])
+    got = _update_zeroed(np.full(11, 2.0), np.zeros(11), 2 * var)[1]
+    assert np.all(np.abs(got - np.sqrt(var)) <= 2.0 ** -23 * np.sqrt(var) + 2.0 ** -148)
+    # infinite and missing sums: the mean follows, a deviation that is no number is 0
+    inf, nan = np.inf, np.nan
+    m, d = _update_zeroed(np.full(4, 4.0), np.array([inf, -inf, nan, 1.0]), np.array([inf, inf, nan, inf]))
+    assert np.array_equal(m, [inf, -inf, nan, 0.25], equal_nan=True) and np.array_equal(d, [0, 0, 0, inf])
