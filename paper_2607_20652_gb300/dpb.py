@@ -293,14 +293,19 @@ def decode(plan: Plan, idx: torch.Tensor, val: torch.Tensor, xnorm=None, y=None,
 
 
 def forward(plan: Plan, x: torch.Tensor, mu=None, sigma=None, workspace=None, stream=None,
-            r_out: Optional[torch.Tensor] = None):
+            r_out: Optional[torch.Tensor] = None, y: Optional[torch.Tensor] = None):
     """dpb_forward (encode then decode). Returns (idx, val, xnorm, y)."""
     _rows(x, plan, "x")
     T, k, dev = x.shape[0], plan.code_len, x.device
     idx = torch.empty((T, k), dtype=torch.int32, device=dev)
     val = torch.empty((T, k), dtype=torch.float32, device=dev)
     xnorm = torch.empty((T,), dtype=torch.float32, device=dev)
-    y = torch.empty_like(x)
+    if y is None:
+        y = torch.empty_like(x)
+    else:
+        _rows(y, plan, "y")
+        if y.shape[0] != T:
+            raise ValueError(f"y must have x's {T} rows")
     if r_out is not None and (r_out.dtype != torch.float32 or not r_out.is_contiguous()
                               or tuple(r_out.shape) != (T, plan.d)):
         raise ValueError(f"r_out must be a contiguous float32 tensor of shape [T, {plan.d}]")

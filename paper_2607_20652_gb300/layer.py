@@ -22,7 +22,9 @@ from . import dpb
 
 class _DPBFunction(torch.autograd.Function):
     # x of any leading shape: the rows are taken here, outside the graph, so
-    # that no reshape node runs in the backward
+    # that no reshape node runs in the backward. y is allocated in x's shape and
+    # written through its rows: the output must not be a view made in here, for
+    # autograd refuses in-place work on such a view (layer(x).add_(x)).
     @staticmethod
     def forward(ctx, x, layer):
         rows = x.reshape(-1, layer.d).contiguous()
@@ -31,7 +33,9 @@ class _DPBFunction(torch.autograd.Function):
         stream = layer._stream(x.device)
         ev = layer._events("forward")
         r = torch.empty((T, layer.d), dtype=torch.float32, device=x.device)  # kept for the backward
-        idx, val, xn, y = dpb.forward(layer.plan, rows, layer.mu, layer.sigma, workspace=ws, stream=stream, r_out=r)
+        y = torch.empty(x.shape, dtype=rows.dtype, device=x.device)
+        idx, val, _, _ = dpb.forward(layer.plan, rows, layer.mu, layer.sigma, workspace=ws, stream=stream, r_out=r,
+                                     y=y.view(T, layer.d))
         if layer.ema is not None and layer.training:
             sample = dpb.sample_rows(T, layer.ema_rows, layer._gen, x.device)
             dpb.stats_accumulate(layer.plan, rows, sample, layer._acc, mu=layer.mu, sigma=layer.sigma, workspace=ws,
@@ -41,7 +45,7 @@ class _DPBFunction(torch.autograd.Function):
         ctx.save_for_backward(rows, idx, val, r)
         ctx.layer = layer
         layer.__dict__["last_code"] = (idx, val)  # (a plain attribute: Module.__setattr__ looks for parameters)
-        return y.view(x.shape)
+        return y
 
     @staticmethod
     def backward(ctx, gy):
