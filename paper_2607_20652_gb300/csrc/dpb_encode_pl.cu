@@ -533,6 +533,12 @@ __device__ __noinline__ void standardise_row(const float *mu, const float *sigma
     if (bad) set_status(status, DPB_DEV_BAD_SIGMA);
 }
 
+// The gathered lists (and half 1's keys) lie in the generator-tile stages, which
+// the producer's bulk copies write next. Those go through the async proxy: each
+// thread's ordinary loads and stores of the lists come before the copies only
+// with this fence between them and the barrier that the producer waits at.
+__device__ __forceinline__ void release_lists() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 // ---- the kernel ----------------------------------------------------------------------
 
 __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
@@ -657,6 +663,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
             wb.par[lane] = 0u;
             __syncwarp();
         }
+        release_lists();
         __syncthreads();
 
         for (int l = 1; l < L && !failed; ++l) {
@@ -855,6 +862,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
                 };
                 select_level(scanl, P, scale, a.kl[l], wb, a, tok, a.off[l], l + 1 < L);
             }
+            release_lists();
             asm volatile("tcgen05.fence::before_thread_sync;");
             __syncthreads();
         }

@@ -171,3 +171,26 @@ def test_wait_that_gives_up_is_flagged_and_leaves_the_context_usable():
         dpb.set_wait_limit(-1)
     assert dpb.workspace_status(ws) & dpb.DEV_TIMEOUT
     _check(plan, ref, kls, x, _gpu(plan, x))
+
+
+@pytest.mark.parametrize("d,bits,children,kls,std", [
+    (1024, [10, 15, 17], [0, 256, 256], [16, 32, 64], False),  # one and two M = 128 tiles a level
+    (2048, [11, 15], [0, 256], [16, 32], True),                # the widest rows, with tables
+    (64, [6, 9, 12], [0, 16, 32], [4, 8, 8], False),           # the gathered lists outgrow the generator tiles
+])
+def test_groups_follow_one_another(d, bits, children, kls, std):
+    # Each block takes several groups of 8 tokens, whose gathered lists and
+    # generator tiles share memory in turn: a row's code is the same bits in
+    # every group, full or partial
+    plan, _ = _plan_ref(d, bits, children, kls)
+    dev = torch.device("cuda")
+    tables = (torch.from_numpy(t).to(dev) for t in inputs.moment_tables(plan.n_features, 5)) if std else (None, None)
+    mu, sigma = tables
+    base = torch.from_numpy(inputs.to_bf16(inputs.gaussian_rows(61, d, 31))).to(dev).to(torch.bfloat16)
+    one = [dpb.encode(plan, base[a:a + 8].contiguous(), mu, sigma) for a in range(0, 61, 8)]
+    want = [torch.cat([o[i] for o in one]) for i in range(3)]
+    for T in (4867, 9733):
+        rows = torch.arange(T, device=dev) % 61
+        for w, o in zip(want, dpb.encode(plan, base[rows].contiguous(), mu, sigma)):
+            assert torch.equal(w[rows], o), T
+    assert plan.status() == 0
