@@ -316,13 +316,14 @@ dpb_status dpb_encode_noalloc(const dpb_plan *plan, const void *x, int64_t T, co
 
 /*
  * dpb_debug_set_wait_limit -- test hook for the bounded waits of the
- * per-level (tcgen05) encoder; the paper has no counterpart. Every
- * mbarrier wait of that kernel's main loop (a generator-tile copy landing,
- * the MMAs of a chunk or level finishing) gives up after `tries` polls for
- * the launches that follow, from any thread; -1 restores the default
- * (2^20 polls). A wait that gives up stops the block: the kernel sets
- * DPB_DEV_TIMEOUT in the workspace status, waits (with the default bound)
- * for its copies and MMAs still in flight, frees its tensor memory and
+ * tensor-core encoders; the paper has no counterpart. Every mbarrier wait of
+ * the per-level (tcgen05) kernel's main loop (a generator-tile copy landing,
+ * the MMAs of a chunk or level finishing), and the global-selection (mma.sync)
+ * kernel's wait for its tables, gives up after `tries` polls for the launches
+ * that follow, from any thread; -1 restores the default (2^20 polls). A wait
+ * that gives up stops the block (the global-selection kernel: the warp): the
+ * kernel sets DPB_DEV_TIMEOUT in the workspace status, waits (with the default
+ * bound) for its copies and MMAs still in flight, frees its tensor memory and
  * returns; that call's codes are incomplete. With tries = 0 every such wait
  * gives up at once, which lets a test exercise that path without a fault.
  * Returns DPB_ERR_INVALID_ARG for tries < -1.

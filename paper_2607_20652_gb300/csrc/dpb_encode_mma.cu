@@ -45,6 +45,7 @@ cudaError_t launch_encode_mma(const dpb_plan *p, const void *x, int64_t T, const
     a.t = p->t;
     a.ecap = mmaenc::entrant_cap(c.k, c.d / 32);
     a.inv_sqrt_d = p->inv_sqrt_d;
+    a.spin = wait_tries();
     const int warps = encode_mma_warps(p);
     const int nkc = std::max(2, p->kvh);
     if (nkc == 2) return mmaenc::launch_nkc2(p, a, warps, stream);

@@ -59,6 +59,7 @@ struct Args {
     int d, nblk, levels, k, t, ecap;
     int beam;  // B <= 8: beam slots B..7 hold no parent
     float inv_sqrt_d;
+    uint32_t spin;  // bound (polls) of the wait for the tables
 };
 
 // ---- shared-memory layout (32-bit words) ------------------------------------------
@@ -124,18 +125,21 @@ __device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t b
                  : "memory");
 }
 
-// Waits (at most 2^20 polls) for the first phase of the mbarrier at `bar`.
-__device__ __forceinline__ bool tables_landed(uint32_t bar) {
-    for (int i = 0; i < 1 << 20; ++i) {
+// Waits (at most `tries` polls) for the first phase of the mbarrier at `bar`.
+// The warp's answer is one: a lane alone would leave the others' shuffles and
+// MMAs without it.
+__device__ __forceinline__ bool tables_landed(uint32_t bar, uint32_t tries) {
+    bool landed = false;
+    for (uint32_t i = 0; i < tries && !landed; ++i) {
         uint32_t done;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
             : "=r"(done)
             : "r"(bar)
             : "memory");
-        if (done) return true;
+        landed = __all_sync(kFull, done != 0u);
     }
-    return false;
+    return landed;
 }
 
 // Parts of parent p's sign words: its Walsh word, the block-parity word
@@ -863,8 +867,12 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
         }
 
         if (!tables) {
-            if (!tables_landed(bar)) {  // never seen: the copies are the block's own
+            if (!tables_landed(bar, a.spin)) {
+                // (never seen at the default bound: the copies are the block's own.)
+                // This warp's codes stay unwritten; it holds the block's shared
+                // memory, again with a bound, until the copies have landed
                 set_status(a.status, DPB_DEV_TIMEOUT);
+                tables_landed(bar, kWaitTries);
                 return;
             }
             tables = true;

@@ -64,7 +64,7 @@ constexpr int kATile = 128 * kChunk * 2;  // one M = 128 tile of a chunk
 constexpr int kSelCap = 256;    // gathered candidates per token and level (up to 8 per lane)
 constexpr int kMaxK = 64;       // K_l per level
 constexpr int kMaxStages = 4;   // generator-tile stages in flight
-constexpr uint32_t kSpin = 1u << 20;  // default bound of the main loop's mbarrier waits, and of the drain
+constexpr uint32_t kSpin = kWaitTries;  // bound of the drain
 // at least this much shared memory per block, so that one block (holding all
 // 512 TMEM columns) runs per SM
 constexpr int kMinSmem = 120 * 1024;
@@ -948,8 +948,8 @@ void build_per_level_tables(dpb_plan *p) {
 
 namespace {
 
-// Bound of the main loop's mbarrier waits for the launches that follow (-1:
-// the default kSpin); set by dpb_debug_set_wait_limit.
+// Bound of the encoders' mbarrier waits for the launches that follow (-1: the
+// default); set by dpb_debug_set_wait_limit.
 std::atomic<int32_t> g_wait_limit{-1};
 
 // Generator-tile stages: as many as fit (at least 2).
@@ -966,6 +966,11 @@ int pl_dmax(const dpb_config &c) {
 }
 
 }  // namespace
+
+uint32_t wait_tries() {
+    const int32_t lim = g_wait_limit.load(std::memory_order_relaxed);
+    return lim < 0 ? kWaitTries : (uint32_t)lim;
+}
 
 size_t encode_pl_smem(const dpb_plan *p) {
     const dpb_config &c = p->cfg;
@@ -1008,8 +1013,7 @@ cudaError_t launch_encode_pl(const dpb_plan *p, const void *x, int64_t T, const 
     }
     a.inv_sqrt_d = p->inv_sqrt_d;
     a.nbs = pl_stages(c, a.kvh, a.dmax);
-    const int32_t lim = g_wait_limit.load(std::memory_order_relaxed);
-    a.spin = lim < 0 ? kSpin : (uint32_t)lim;
+    a.spin = wait_tries();
     const size_t smem = encode_pl_smem(p);
     const cudaError_t e = allow_smem((const void *)encode_pl_kernel, smem);
     if (e != cudaSuccess) return e;

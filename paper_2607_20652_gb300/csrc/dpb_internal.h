@@ -100,6 +100,12 @@ int encode_mma_warps(const dpb_plan *p);
 size_t encode_mma_smem(const dpb_plan *p, int warps);
 constexpr size_t kMaxSmemPerBlock = 227 * 1024;
 
+// Bounded mbarrier waits of the encoders: the default number of polls (also of
+// the drain after a wait has given up), and the number for the launches that
+// follow (dpb_debug_set_wait_limit).
+constexpr uint32_t kWaitTries = 1u << 20;
+uint32_t wait_tries();
+
 // Lets kernel `func` use `bytes` of dynamic shared memory on the current
 // device. The attribute is set the first time a kernel needs more than its
 // default (and again only when a later launch needs more), so repeated

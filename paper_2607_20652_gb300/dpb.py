@@ -406,8 +406,8 @@ def stats_step(plan: Plan, x: torch.Tensor, mu: torch.Tensor, sigma: torch.Tenso
 
 
 def set_wait_limit(tries: int = -1):
-    """dpb_debug_set_wait_limit: bound of the per-level encoder's main-loop
-    mbarrier waits for the launches that follow (-1 restores the default)."""
+    """dpb_debug_set_wait_limit: bound of the tensor-core encoders' mbarrier
+    waits for the launches that follow (-1 restores the default)."""
     _check(load().dpb_debug_set_wait_limit(int(tries)))
 
 

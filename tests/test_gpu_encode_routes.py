@@ -82,3 +82,24 @@ def test_rows_do_not_depend_on_their_batch(beam, k, std):
         for w, o in zip(want, out):
             assert torch.equal(w[rows], o), T
     assert plan.status() == 0
+
+
+@pytest.mark.parametrize("T", [1, 37, 5000])
+def test_table_wait_that_gives_up_is_flagged(T):
+    """With the wait for the tables bounded at 0 polls the tensor-core encoder
+    flags DPB_DEV_TIMEOUT, lets its copies land and returns; the next call is
+    whole again."""
+    plan = dpb.Plan(d=96, levels=4, m_bits=14, children=16, beam=8, k=64, dtype="bf16")
+    x = torch.from_numpy(inputs.gaussian_rows(T, 96, 8)).cuda().to(torch.bfloat16)
+    want = dpb.encode(plan, x)
+    assert plan.status() == 0
+    try:
+        dpb.set_wait_limit(0)
+        dpb.encode(plan, x)
+        torch.cuda.synchronize()
+    finally:
+        dpb.set_wait_limit(-1)
+    assert plan.status() == dpb.DEV_TIMEOUT
+    for w, o in zip(want, dpb.encode(plan, x)):
+        assert torch.equal(w, o)
+    assert plan.status() == 0
