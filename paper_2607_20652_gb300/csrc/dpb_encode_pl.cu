@@ -761,7 +761,10 @@ __global__ void __launch_bounds__(kThreads, 1) encode_pl_kernel(Args a) {
                 // MMAs of chunk c - na are done (a stage of an earlier level is free)
                 for (int c = 0; c < nch; ++c) {
                     const uint32_t g = G0 + c;
-                    if (c >= na && !mbar_wait(mma_done(g - na), phase(g - na), a.spin)) {
+                    // (the warp gives up as one: a lane alone would leave the others
+                    // at the __syncwarp below)
+                    const bool free_stage = c < na || mbar_wait(mma_done(g - na), phase(g - na), a.spin);
+                    if (!__all_sync(kFull, free_stage)) {
                         bfail = true;
                         break;
                     }

@@ -194,3 +194,24 @@ def test_groups_follow_one_another(d, bits, children, kls, std):
         for w, o in zip(want, dpb.encode(plan, base[rows].contiguous(), mu, sigma)):
             assert torch.equal(w[rows], o), T
     assert plan.status() == 0
+
+
+@pytest.mark.parametrize("tries", [0, 1, 2, 8])
+def test_waits_that_give_up_anywhere_end(tries):
+    # Bounds at which some waits of the main loop give up and others (other warps',
+    # other chunks') do not: the call ends, a code is flagged or whole, and the
+    # next call is whole
+    plan, _ = _plan_ref(1024, [10, 15, 17], [0, 256, 256], [16, 32, 64])
+    x = torch.from_numpy(inputs.to_bf16(inputs.gaussian_rows(2500, 1024, 32))).cuda().to(torch.bfloat16)
+    want = dpb.encode(plan, x)
+    assert plan.status() == 0
+    try:
+        dpb.set_wait_limit(tries)
+        got = dpb.encode(plan, x)
+        torch.cuda.synchronize()
+    finally:
+        dpb.set_wait_limit(-1)
+    status = plan.status()
+    assert status == dpb.DEV_TIMEOUT or (status == 0 and all(map(torch.equal, want, got)))
+    assert all(map(torch.equal, want, dpb.encode(plan, x)))
+    assert plan.status() == 0
