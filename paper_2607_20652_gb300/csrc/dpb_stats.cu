@@ -398,17 +398,21 @@ __global__ void __launch_bounds__(kSearchThreads, 1) stats_search_kernel(StatsAr
 
 // ---- the EMA step -----------------------------------------------------------------
 
-// 1 / n, a / n and sqrt(v) in fp64 by Newton's iteration from an fp32 estimate
-// (an error of 2^-22 squares to 2^-44 and then below fp64's): this chip has about
-// two fp64 lanes per SM and clock, and the library's division and root take some
-// 120 fp64 instructions a feature where these take 25.
+// a / n and sqrt(v) in fp64: one step of Newton's iteration from an fp32 estimate
+// (an error of 2^-22 squares to 2^-44), then the result corrected by its
+// remainder (squared again, below fp64's rounding). This chip has about two fp64
+// lanes per SM and clock, and the library's division and root take some 120 fp64
+// instructions a feature where these take 20. Their ranges are tested on the high
+// words, off the fp64 pipe.
+constexpr int kHi2m99 = 0x39C00000, kHi2p99 = 0x46200000;  // high words of 2^-99 and 2^99
+constexpr int kHiHalf = 0x3FE00000, kHi1p5 = 0x3FF80000;    // and of 1/2 and 3/2
+
+// 1 / n to 2^-44 (0.5 <= n < 2^99)
 __device__ __forceinline__ double newton_rcp(double n) {
-    if (!(n < 1e30)) return 1.0 / n;  // (fp32's range)
-    double r = (double)(1.0f / (float)n);
-    r = fma(r, fma(-n, r, 1.0), r);
+    const double r = (double)(1.0f / (float)n);
     return fma(r, fma(-n, r, 1.0), r);
 }
-// a / n with rn = 1 / n: the remainder of the rounded product corrects it to the
+// a / n with rn near 1 / n: the remainder of the rounded product corrects it to the
 // quotient rounded once. The variance q / n - (s / n)^2 cancels, so a second
 // rounding is not lost in the fp32 result: with plain products one feature in
 // fifteen whose scores are all equal got a deviation of up to 2e-8 of its mean
@@ -416,15 +420,29 @@ __device__ __forceinline__ double newton_rcp(double n) {
 // and NaN go past the remainder, which would turn the first into the second.
 __device__ __forceinline__ double quotient(double a, double n, double rn) {
     const double q = a * rn;
-    return isfinite(q) ? fma(fma(-n, q, a), rn, q) : q;
+    return (__double2hiint(q) & 0x7FF00000) != 0x7FF00000 ? fma(fma(-n, q, a), rn, q) : q;
 }
-__device__ __forceinline__ double newton_sqrt(double v) {
-    if (!(v > 1e-30 && v < 1e30)) return sqrt(v);  // outside fp32's comfortable range
-    double r = (double)rsqrtf((float)v);           // r -> 1 / sqrt(v): r += r (1 - v r^2) / 2
-    r = fma(0.5 * r, fma(-v * r, r, 1.0), r);
+// The library's root where the fast one does not reach; a call, like
+// ema_unusual, so that its code takes no registers of the kernel.
+__device__ __noinline__ double root_unusual(double v) { return sqrt(v); }
+// sqrt(max(v, 0)), 0 for NaN
+__device__ __forceinline__ double root(double v) {
+    if ((uint32_t)(__double2hiint(v) - kHi2m99) >= (uint32_t)(kHi2p99 - kHi2m99)) return v > 0.0 ? root_unusual(v) : 0.0;
+    double r = (double)rsqrtf((float)v);  // r -> 1 / sqrt(v): r += r (1 - v r^2) / 2
     r = fma(0.5 * r, fma(-v * r, r, 1.0), r);
     const double y = v * r;
     return fma(0.5 * r, fma(-y, y, v), y);
+}
+
+// The step for a count that is none (NaN, or 2^99 and more); a call, so that the
+// library's division and root take no registers of the kernel.
+__device__ __noinline__ void ema_unusual(double n, double s, double q, double alpha, float *mu, float *sigma) {
+    const double mean = s / n, mu0 = *mu;
+    *mu = (float)(mu0 + alpha * (mean - mu0));
+    if (n >= 1.5) {
+        const double sg0 = *sigma;
+        *sigma = (float)(sg0 + alpha * (root(q / n - mean * mean) - sg0));
+    }
 }
 
 // A block reads the counts of kUpdFeatures features and lists the touched ones,
@@ -434,10 +452,13 @@ __device__ __forceinline__ double newton_sqrt(double v) {
 // arithmetic to one SM. 2^20 features, 3% touched: 16.8 us with a feature per
 // thread and library arithmetic; the standardised step of 8,192 tokens 298 us
 // with blocks of 1,024 and library arithmetic, 284 with blocks of 512 and 282
-// with 256 of these.
+// with 256 and Newton arithmetic. 8 blocks to an SM (32 registers): 2^20
+// features, none, 3%, half and all of them touched 8.0, 16.4, 39.6 and 63.6 us,
+// with the 44 registers of no bound 8.6, 19.5, 40.8 and 63.6 (a feature per
+// thread and library arithmetic 9.4, 51.8, 75.9 and 75.9).
 constexpr int kUpdFeatures = 256;
-__global__ void __launch_bounds__(256) stats_update_kernel(double *acc, int64_t m, double alpha, float *mu,
-                                                           float *sigma) {
+__global__ void __launch_bounds__(256, 8) stats_update_kernel(double *acc, int64_t m, double alpha, float *mu,
+                                                              float *sigma) {
     __shared__ uint16_t list[kUpdFeatures];
     __shared__ int count;
     for (int64_t base = (int64_t)blockIdx.x * kUpdFeatures; base < m; base += (int64_t)gridDim.x * kUpdFeatures) {
@@ -456,15 +477,17 @@ __global__ void __launch_bounds__(256) stats_update_kernel(double *acc, int64_t 
         for (int e = threadIdx.x; e < count; e += 256) {
             const int64_t i = base + list[e];
             const double n = acc[i], s = acc[m + i], q = acc[2 * m + i];
-            const double rn = newton_rcp(n);
-            const double mean = quotient(s, n, rn);
-            const double mu0 = mu[i];
-            mu[i] = (float)(mu0 + alpha * (mean - mu0));
-            if (n >= 1.5) {
-                const double var = quotient(q, n, rn) - mean * mean;
-                const double v = var > 0.0 ? newton_sqrt(var) : 0.0;
-                const double sg0 = sigma[i];
-                sigma[i] = (float)(sg0 + alpha * (v - sg0));
+            const int hn = __double2hiint(n);
+            if ((uint32_t)(hn - kHiHalf) < (uint32_t)(kHi2p99 - kHiHalf)) {
+                const double rn = newton_rcp(n), mean = quotient(s, n, rn);
+                const double mu0 = mu[i];
+                mu[i] = (float)(mu0 + alpha * (mean - mu0));
+                if (hn >= kHi1p5) {
+                    const double sg0 = sigma[i];
+                    sigma[i] = (float)(sg0 + alpha * (root(quotient(q, n, rn) - mean * mean) - sg0));
+                }
+            } else {
+                ema_unusual(n, s, q, alpha, mu + i, sigma + i);
             }
             acc[i] = 0.0;
             acc[m + i] = 0.0;
