@@ -498,15 +498,29 @@ __global__ void __launch_bounds__(256, 8) stats_update_kernel(double *acc, int64
 }
 
 template <typename Tio>
-cudaError_t run_columns(const Tio *x, int64_t T, int d, double *acc, int64_t m, cudaStream_t stream) {
-    // enough blocks for the chip on a batch of a few thousand rows; on a large
-    // one half the atomics
-    const int rows = T <= 16384 ? 4 * kColChunk : 8 * kColChunk;
-    const dim3 grid((unsigned)((T + rows - 1) / rows), (unsigned)((d + kColThreads - 1) / kColThreads));
-    if (d % 4 == 0)  // (x is 16-byte aligned)
-        stats_columns_kernel<Tio, 4><<<grid, kColThreads, 0, stream>>>(x, T, d, rows, acc, m);
+cudaError_t run_columns(const dpb_plan *p, const Tio *x, int64_t T, double *acc, int64_t m, cudaStream_t stream) {
+    const int d = p->cfg.d, cols = (d + kColThreads - 1) / kColThreads;
+    // fp32 rows of more than 256 columns: a column a thread already reads whole
+    // 128-byte lines, and four took 45 us where one takes 37 (65,536 x 768, out of
+    // DRAM; 32 and 25 at 16,384 x 2,048). bf16 rows, and narrow fp32 ones, four:
+    // 65,536 x 768 bf16 29 us, with one 31; 65,536 x 100 fp32 17 and 21.
+    const bool one = d % 4 != 0 || (sizeof(Tio) == 4 && cols > 1);  // (x is 16-byte aligned)
+    int64_t rows;  // of a block
+    if (sizeof(Tio) == 4 && cols > 1) {
+        // the fewest with every block resident (8 to an SM): half as many rows
+        // take 43 us at 65,536 x 768, twice as many 52
+        rows = kColChunk;
+        while ((T + rows - 1) / rows * cols > 8ll * std::max(p->sms, 1)) rows *= 2;
+    } else {
+        // 16,384 x 768 bf16: 12.6 us with 128 rows, 14.6 with 256 (too few blocks);
+        // 32,768: 20.8 and 18.6 (atomics)
+        rows = T <= 16384 ? 4 * kColChunk : 8 * kColChunk;
+    }
+    const dim3 grid((unsigned)((T + rows - 1) / rows), (unsigned)cols);
+    if (one)
+        stats_columns_kernel<Tio, 1><<<grid, kColThreads, 0, stream>>>(x, T, d, (int)rows, acc, m);
     else
-        stats_columns_kernel<Tio, 1><<<grid, kColThreads, 0, stream>>>(x, T, d, rows, acc, m);
+        stats_columns_kernel<Tio, 4><<<grid, kColThreads, 0, stream>>>(x, T, d, (int)rows, acc, m);
     return cudaGetLastError();
 }
 
@@ -557,8 +571,8 @@ cudaError_t launch_stats_accumulate(const dpb_plan *p, const void *x, int64_t T,
     const int64_t m = (int64_t)p->m_mask + 1;
     if (T > 0) {
         const cudaError_t e = p->cfg.dtype == DPB_BF16
-                                  ? run_columns(static_cast<const __nv_bfloat16 *>(x), T, d, acc, m, stream)
-                                  : run_columns(static_cast<const float *>(x), T, d, acc, m, stream);
+                                  ? run_columns(p, static_cast<const __nv_bfloat16 *>(x), T, acc, m, stream)
+                                  : run_columns(p, static_cast<const float *>(x), T, acc, m, stream);
         if (e != cudaSuccess) return e;
     }
     if (n_sample == 0 || p->cfg.levels < 2) return cudaSuccess;

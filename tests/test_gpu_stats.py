@@ -343,3 +343,20 @@ def test_ema_update_deviations_against_exact_arithmetic():
     inf, nan = np.inf, np.nan
     m, d = _update_zeroed(np.full(4, 4.0), np.array([inf, -inf, nan, 1.0]), np.array([inf, inf, nan, inf]))
     assert np.array_equal(m, [inf, -inf, nan, 0.25], equal_nan=True) and np.array_equal(d, [0, 0, 0, inf])
+
+
+@pytest.mark.parametrize("T,d,dtype", [
+    (1, 260, "f32"), (33, 257, "f32"),          # a column a thread, a partial second column block
+    (19456, 260, "f32"), (19457, 260, "f32"),   # the last batch with 32 rows a block, the first with 64
+    (20000, 256, "f32"), (129, 260, "bf16"),    # four columns a thread
+    (16384, 64, "bf16"), (16385, 64, "bf16"),   # 128 and 256 rows a block
+])
+def test_column_sums_over_the_shapes_of_their_launch(T, d, dtype):
+    plan, _ = _pair(dtype=dtype, d=d, levels=3, m_bits=14, children=16, beam=4, k=8)
+    x = torch.randn((T, d), generator=torch.Generator().manual_seed(29)).cuda().to(plan.torch_dtype)
+    acc = dpb.stats_buffer(plan)
+    dpb.stats_accumulate(plan, x, torch.empty(0, dtype=torch.int32, device="cuda"), acc)
+    v = x.double()
+    assert bool((acc[0, :d] == T).all()) and not acc[:, d:].any().item()
+    for got, want, bound in ((acc[1, :d], v.sum(0), v.abs().sum(0)), (acc[2, :d], v.square().sum(0), v.square().sum(0))):
+        assert bool(((got - want).abs() <= 1e-5 * bound + 1e-30).all())
