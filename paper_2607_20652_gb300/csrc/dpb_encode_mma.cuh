@@ -142,6 +142,16 @@ __device__ __forceinline__ bool tables_landed(uint32_t bar, uint32_t tries) {
     return landed;
 }
 
+// The same as a call, with what follows when the wait gives up: the warp's codes
+// stay unwritten, and it holds the block's shared memory, again with a bound,
+// until the copies have landed.
+static __device__ __noinline__ bool tables_landed_call(uint32_t bar, uint32_t tries, int32_t *status) {
+    if (tables_landed(bar, tries)) return true;
+    set_status(status, DPB_DEV_TIMEOUT);
+    tables_landed(bar, kWaitTries);
+    return false;
+}
+
 // Parts of parent p's sign words: its Walsh word, the block-parity word
 // (bit m = parity(m AND u), u = bits 5..9 of p_lo: the Walsh word of u) and
 // the byte offsets into VH_k[m], packed to a word.
@@ -794,10 +804,10 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
     }
     if (COSET)
         for (int i = threadIdx.x; i < (L - 1) * (nblk + 16); i += blockDim.x) s_frag[i] = a.coset[i];
-    for (int v = threadIdx.x; v < 32; v += blockDim.x) {
+    if (threadIdx.x < 32) {
         uint32_t word = 0;
-        for (int l = 0; l < 32; ++l) word |= (uint32_t)(__popc(l & v) & 1) << l;
-        s_w5[v] = word;
+        for (int l = 0; l < 32; ++l) word |= (uint32_t)(__popc(l & threadIdx.x) & 1) << l;
+        s_w5[threadIdx.x] = word;
     }
     for (int i = threadIdx.x; i < L * 16; i += blockDim.x) s_g[i] = a.G[(i >> 4) * DPB_MAX_CHILDREN + (i & 15)];
     __syncthreads();
@@ -867,10 +877,13 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
         }
 
         if (!tables) {
-            if (!tables_landed(bar, a.spin)) {
-                // (never seen at the default bound: the copies are the block's own.)
-                // This warp's codes stay unwritten; it holds the block's shared
-                // memory, again with a bound, until the copies have landed
+            // (never given up at the default bound: the copies are the block's own.)
+            // A call, except for lists of 33 to 64 words, where the kernel's code
+            // around it comes out slower: 65,536 tokens at k = 64 540 us in place and
+            // 544 with the call, at k = 32 405 and 398, 32,768 at k = 128 326 and 317
+            if constexpr (WIDE || KPL != 2) {
+                if (!tables_landed_call(bar, a.spin, a.status)) return;
+            } else if (!tables_landed(bar, a.spin)) {
                 set_status(a.status, DPB_DEV_TIMEOUT);
                 tables_landed(bar, kWaitTries);
                 return;
@@ -1083,10 +1096,14 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) encode_kernel(Args a) {
                 }
                 pcur = p1;
                 const bool next = l + 1 < L;
-                // the merge in place, except for lists of 33 to 64 words, whose
-                // loop the call keeps small: 65,536 tokens forward at k = 64 took 670
-                // us with the call and 679 without, at k = 128 1,060 and 1,031, and
-                // the sweep step at beam 16, k = 128 1,144 and 1,093
+                // the merge in place, except for lists of 33 to 64 words with two
+                // tokens a warp, whose loop the call keeps small. Encode, us in place
+                // and with the call: two tokens, 65,536 at k = 16 471 and 478, 32 498
+                // and 500, 64 679 and 670 (with the decode), 128 675 and 678; 16,384 at
+                // k = 200 897 and 908, 256 955 and 961. Beam 16: 65,536 at k = 16 909
+                // and 965, 32 938 and 1,001, 64 1,015 and 1,082, 128 1,204 and 1,327;
+                // 16,384 at k = 200 1,072 and 1,099, 256 1,118 and 1,128 (with tables
+                // 1,133 and 1,126, 1,370 and 1,364)
                 const int m = merge_entrants<KPL, WIDE || KPL != 2>(Lt, k, E, c, next && !WIDE ? bt : nullptr);
                 if constexpr (WIDE) {
                     if (tk == 0) {
