@@ -161,7 +161,8 @@ dpb_status dpb_code_length(const dpb_plan *plan, int32_t *k_out);
 /* Bytes of workspace for T tokens (256-byte aligned pointer required): 256
  * bytes for the device status word, then 8 * 2^N bytes (for 2^N <= 2^26)
  * where dpb_encode packs the standardisation tables as (mu, 1 / sigma) pairs,
- * so that each candidate costs one table load instead of two. Any workspace of
+ * so that each candidate costs one table load instead of two (the tensor-core
+ * encoders; the others read the two tables and leave these bytes unused). Any workspace of
  * at least 256 bytes is accepted; a smaller one than this size only leaves the
  * tables unpacked (same results, slower with tables). The status word must be
  * zero-filled once before its first use; the workspace may be reused by every

@@ -241,10 +241,10 @@ __device__ __forceinline__ void add_block(float2 &acc, const uint32_t *vh2, int 
 // gv[p] += sum_i h[i] (-1)^{parity(M[i] AND hc_p)} for the nh hashed codes.
 // Per chunk of 4 blocks: nibble tables TH[b][n][v] = sum_j (-1)^{v_j}
 // h[32b + 4n + j] (16 entries per 4 coordinates); a code's sign word over a
-// block indexes that block's 8 tables. The first nh - nh % 32 codes go one
-// per lane through all blocks of the chunk; each of the others gets 4 lanes,
-// one block each, summed by shuffles. Every code's sum is taken in a fixed
-// order.
+// block indexes that block's 8 tables. Whole 32s of codes, and a remainder of
+// more than kTail, go one per lane through all blocks of the chunk; a code of a
+// smaller remainder gets 4 lanes, one block each, summed by shuffles. Every
+// code's sum is taken in a fixed order.
 template <int NKC>
 __device__ __forceinline__ void analyse(const BwdWarp &w, int nh, int d, const uint32_t *vh2) {
     const int lane = threadIdx.x & 31;
@@ -421,8 +421,8 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2) backward_lut_kernel(Backwar
             __syncwarp();
         }
         // Two synthesis passes share one call site: pass 0 builds r (norm
-        // matching only) and turns it into dL/dr; pass 1 adds the hashed
-        // entries' sum to grad_x.
+        // matching only) and turns it into dL/dr; pass 1 takes grad_val from it
+        // and overwrites it with the hashed entries' part of grad_x.
 #pragma unroll 1
         for (int pass = !kept_r && a.norm_match ? 0 : 1;; ++pass) {
             if (pass == 1) {

@@ -94,8 +94,8 @@ cudaError_t launch_encode_pl(const dpb_plan *p, const void *x, int64_t T, const 
                              const float2 *tab, int32_t *idx, float *val, float *xnorm, int32_t *status,
                              cudaStream_t stream);
 
-// Launch shape of the tensor-core encoder: the most warps per block (16, 12,
-// 8 or 4) whose shared memory fits, or 0 if none does; and that memory.
+// Launch shape of the tensor-core encoder: the most warps per block (20, 16,
+// 12, 8 or 4) whose shared memory fits, or 0 if none does; and that memory.
 int encode_mma_warps(const dpb_plan *p);
 size_t encode_mma_smem(const dpb_plan *p, int warps);
 constexpr size_t kMaxSmemPerBlock = 227 * 1024;
@@ -157,7 +157,9 @@ cudaError_t launch_encode(const dpb_plan *p, const void *x, int64_t T, const flo
 
 // Workspace: the status word (kStatusBytes, required) and, after it, the
 // optional packed standardisation tables (8 bytes per feature, for 2^N up to
-// 2^26; 0 bytes beyond).
+// 2^26; 0 bytes beyond). The size is the same for every plan; the encoders
+// outside the tensor cores (dpb_encode_fma.cu, dpb_encode.cu) read mu and sigma
+// from the two tables, with a true division, and leave these bytes unused.
 constexpr size_t kStatusBytes = 256;
 inline size_t tab_bytes(const dpb_plan *p) {
     const uint64_t m = (uint64_t)p->m_mask + 1;
