@@ -13,9 +13,10 @@
 // index 2 lane + e = 16 slot + j). Every sum is taken in the order of a
 // per-child lane sum followed by an xor butterfly (o = 16, 8, ..., 1).
 //
-// What bounds it: issue and L1, about 70 instructions and 18 L1 wavefronts per
-// 32 coordinates and 4 parents, and with few tokens a token's own chain of
-// levels. Measured, encode and decode of 3,001 fp32 rows (d = 768, 4 levels,
+// What bounds it: the latency of the table loads and of a token's own chain at 12
+// warps per SM (168 registers): about 70 instructions and 18 L1 wavefronts per 32
+// coordinates and 4 parents, 41% of the cycles issue, L1 a third of its
+// wavefronts. Measured, encode and decode of 3,001 fp32 rows (d = 768, 4 levels,
 // beam 8, k = 32): 97 us, where a popcount per (child, coordinate), a warp sum
 // per child and selection by bisection took 552 us; 256 rows of d = 64 (3
 // levels, beam 4, k = 8): 71 to 15 us.
